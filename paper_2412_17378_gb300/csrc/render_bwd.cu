@@ -170,7 +170,7 @@ __device__ __forceinline__ void warp_reduce_red(const PairSums &s, float dx, flo
 }
 
 // Record of list entry j and its index g; an index >= N raises BGS_CHECK_INDEX and yields a
-// transparent record (its box misses every pixel) with index 0.
+// transparent record (its level misses every pixel) with index 0.
 __device__ __forceinline__ Rec load_rec_bwd(const BwdArgs &a, uint32_t j, uint32_t &g) {
     g = a.point_list[j];
     Rec r;
@@ -178,7 +178,7 @@ __device__ __forceinline__ Rec load_rec_bwd(const BwdArgs &a, uint32_t j, uint32
         raise_check(a.ctrl, BGS_CHECK_INDEX);
         g = 0;
         r.a = make_float4(0.f, 0.f, 0.f, 0.f);
-        r.b = make_float4(0.f, 0.f, -1.f, -1.f);
+        r.b = make_float4(0.f, 0.f, -3.0e38f, 0.f);
         r.c = make_float4(0.f, 0.f, 0.f, 0.f);
         return r;
     }
@@ -339,9 +339,9 @@ __device__ __forceinline__ void bwd_pixel_item(const BwdArgs &a, int tile, int s
             const Rec r = load_rec_bwd(a, top - 1 - lane, g);
             buf[lane] = r;
             gbuf[lane] = g;
-            hit = !box_misses(r.a, r.b, bcx, bcy, 0.5f * (kItemW - 1), 0.5f * (kItemH - 1));
+            hit = !block_misses(r.a, r.b, bcx, bcy, 0.5f * (kItemW - 1), 0.5f * (kItemH - 1));
         }
-        // back to front over the records whose alpha box reaches the pixel block
+        // back to front over the records that can reach alpha >= 1/255 in the pixel block
         unsigned live = __ballot_sync(kFullB, hit);
         __syncwarp();
         while (live) {

@@ -66,8 +66,8 @@ __device__ __forceinline__ Rec load_rec(const FwdArgs &a, uint32_t j) {
         raise_check(a.ctrl, BGS_CHECK_INDEX);
         Rec r;
         r.a = make_float4(0.f, 0.f, 0.f, 0.f);
-        r.b = make_float4(0.f, 0.f, 0.f, 0.f);
-        r.c = r.b;
+        r.b = make_float4(0.f, 0.f, -3.0e38f, 0.f);
+        r.c = r.a;
         return r;
     }
     return a.recs[g];
@@ -221,9 +221,9 @@ __device__ __forceinline__ void pixel_item(const FwdArgs &a, int tile, int sub, 
         if (j < rg.y) {
             const Rec r = load_rec(a, j);
             buf[lane] = r;
-            hit = !box_misses(r.a, r.b, bcx, bcy, 0.5f * (kItemW - 1), 0.5f * (kItemH - 1));
+            hit = !block_misses(r.a, r.b, bcx, bcy, 0.5f * (kItemW - 1), 0.5f * (kItemH - 1));
         }
-        // records whose alpha box reaches the item's pixel block; the others are skipped
+        // records that can reach alpha >= 1/255 in the item's pixel block; the others are skipped
         unsigned live = __ballot_sync(kFull, hit);
         __syncwarp();
         const int pos0 = (int)(base - rg.x);
