@@ -76,11 +76,12 @@ __host__ __device__ constexpr int pix_row_step(int Q) { return 32 / pix_item_w(Q
 __host__ __device__ constexpr int pix_item_h(int Q) { return pix_row_step(Q) * Q; }
 
 // ---- packed per-Gaussian record used by the render kernels (48 bytes) ---------------
-//   a = (mx, my, qa, qb), b = (qc, o, lv, 0), c = (r, g, b, depth)
+//   a = (mx, my, qa, qb), b = (qc, o, lv, odd), c = (r, g, b, depth)
 //   with (qa, qb, qc) = -log2(e) (a/2, b, c/2), so that the natural-log power of the
 //   pair is ln2 * (qa dx^2 + qb dx dy + qc dy^2) and exp(power) = 2^(qa dx^2 + ...).
 //   A pair reaches alpha >= 1/255 only where that exponent is at least -lv (see
-//   alpha_level); kernels use it to skip whole records for a block of pixels.
+//   alpha_level); kernels use it to skip whole records for a block of pixels.  odd is not
+//   0 for the records that need the pair rule in full (record_odd).
 struct __align__(16) Rec {
     float4 a, b, c;
 };
@@ -115,6 +116,20 @@ __device__ __forceinline__ float alpha_level(float a, float b, float c, float o)
     return a * c - b * b > 0.f ? log2f(lo) : 3.0e38f;
 }
 
+// 0 times x is 0, and no product of two such values overflows (false for infinities and NaN).
+__device__ __forceinline__ bool tame(float x) { return fabsf(x) < 1e18f; }
+
+// 0 when, at every pixel, the clamp and the sign test of the pair rule decide nothing and a
+// masked pair adds nothing: o <= 0.99 (so o G is); the exponent is never above 0 by rounding
+// (its float32 error is below 4e-7 of the sum of its square terms, which at det >= 1e-5 a c
+// exceed the cross term by 5e-6 of it); and colour and depth are tame.  2 when they are not, 1
+// for the other records.
+__device__ __forceinline__ float record_odd(float a, float b, float c, float o, float4 rgbd) {
+    const float ac = a * c;
+    if (!(tame(rgbd.x) && tame(rgbd.y) && tame(rgbd.z) && tame(rgbd.w))) return 2.f;
+    return o <= kAlphaMax && a > 0.f && ac < 1e30f && ac - b * b >= 1e-5f * ac ? 0.f : 1.f;
+}
+
 // Packs record g into a Rec (the conic is pre-scaled by -log2(e)/2); its colour is
 // colour row cg (views of a batched call share the colours of their Gaussians).
 __device__ __forceinline__ Rec make_rec(const float *__restrict__ means2D, const float *__restrict__ conic_opacity,
@@ -124,8 +139,9 @@ __device__ __forceinline__ Rec make_rec(const float *__restrict__ means2D, const
     const float2 m = reinterpret_cast<const float2 *>(means2D)[g];
     const float4 co = reinterpret_cast<const float4 *>(conic_opacity)[g];
     r.a = make_float4(m.x, m.y, -0.5f * kLog2e * co.x, -kLog2e * co.y);
-    r.b = make_float4(-0.5f * kLog2e * co.z, co.w, alpha_level(co.x, co.y, co.z, co.w), 0.f);
     r.c = make_float4(colors[3 * cg], colors[3 * cg + 1], colors[3 * cg + 2], depths[g]);
+    r.b = make_float4(-0.5f * kLog2e * co.z, co.w, alpha_level(co.x, co.y, co.z, co.w),
+                      record_odd(co.x, co.y, co.z, co.w, r.c));
     return r;
 }
 
@@ -202,6 +218,36 @@ __device__ __forceinline__ float next_T(float T, float al) { return __fmaf_rn(-T
 // o G of a pair.  A pair is accumulated when power2 <= 0 and o G >= 1/255 (the same as
 // alpha = min(0.99, o G) >= 1/255, since 1/255 < 0.99); alpha is formed only for those.
 __device__ __forceinline__ float pair_oG(float power2, float o) { return __fmul_rn(o, ex2_approx(power2)); }
+
+// ---- pairs of float32 values in one 64-bit register (both halves rounded like the scalar
+// instruction; one issue slot for two results) --------------------------------------------
+typedef unsigned long long F2;
+
+__device__ __forceinline__ F2 f2(float lo, float hi) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 f2_split(F2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
 
 // ---- views ---------------------------------------------------------------------------
 // A render call covers V views (1 for the single-view entry points).  Their tiles form
