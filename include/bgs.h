@@ -104,8 +104,8 @@ typedef struct bgs_plan_desc {
                                 walked by separate warps, and a merge pass composes each
                                 pixel's segments (its stop taken by the sequential rule); the
                                 split is skipped (one segment per tile) when it would need more
-                                than 2^24 items or one per (segment, pixel group) over
-                                num_entries / gw_segment segments                           */
+                                than num_entries / gw_segment + 1 segments after the tiles'
+                                first ones, or 2^24 pixel groups over them                  */
 } bgs_plan_desc;
 
 typedef struct bgs_plan bgs_plan;

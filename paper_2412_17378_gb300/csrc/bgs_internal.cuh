@@ -23,7 +23,7 @@ struct DevCtrl {
     unsigned int queue_head;    // pixel-wise queue cursor (starts at num_gauss)
     unsigned int num_items;     // work items in the current list
     unsigned int check_bits;    // BGS_CHECK_* raised by device checks
-    unsigned int num_gauss;     // items [0, num_gauss) are Gaussian-wise, the rest pixel-wise
+    unsigned int num_gauss;     // item numbers [0, num_gauss) are Gaussian-wise, the rest pixel-wise
     unsigned long long num_entries;  // K written by binning
     unsigned long long eval_pairs;
     unsigned long long contrib_pairs;
@@ -38,11 +38,11 @@ struct DevCtrl {
     unsigned int wl_cnt[256];
     unsigned int wl_off[256];
     unsigned int wl_done;
-    unsigned int num_gauss0;    // Gaussian-wise items [0, num_gauss0) are first segments; the
-                                // items [num_gauss0, num_gauss) later segments of long lists
+    unsigned int gw_first;      // Gaussian-wise segments [0, gw_first) are the tiles' first ones;
+                                // the later ones of long lists follow
     unsigned int gw_seg;        // entries per Gaussian-wise segment (0: lists are not split)
-    unsigned int pad2;
-    unsigned long long wl_extra;  // work-list build: later-segment items (returns to zero)
+    unsigned int gw_wide;       // the segments' items: blocks of pixels (1) or pixel groups (0)
+    unsigned long long wl_extra;  // work-list build: later segments (returns to zero)
     // binning: each view's entry count and first point_list slot
     unsigned long long view_k[kMaxViews];
     unsigned long long view_base[kMaxViews];
@@ -86,9 +86,15 @@ struct __align__(16) Rec {
     float4 a, b, c;
 };
 
-// One work item of the persistent kernels.
-//   x = tile id (global over views), y = kind << 31 | sub-item index inside the tile.
-constexpr unsigned int kKindGauss = 1u << 31;
+// One pixel-wise work item of the persistent kernels: x = tile id (global over views), y =
+// sub-item index inside the tile.  Gaussian-wise tiles have one entry per segment of their
+// list instead, (tile id, segment), whose items are numbered arithmetically (gw_items_per):
+// kGwBlock x kGwBlock blocks of the tile's pixels, or groups of gw_pixels pixels.
+constexpr int kGwBlock = 8;
+
+__host__ __device__ constexpr int gw_blocks_per(int tile_w, int tile_h) {
+    return ((tile_w + kGwBlock - 1) / kGwBlock) * ((tile_h + kGwBlock - 1) / kGwBlock);
+}
 
 // ---- small device helpers ------------------------------------------------------------
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -295,18 +301,20 @@ struct FwdArgs {
     ViewTable vt;
     ViewOut io;
     DevCtrl *ctrl;
-    const uint2 *items;          // work list (persistent kernels)
-    int pass_blocks;             // blocks of the persistent pass (both forward kernels when both run)
+    const uint2 *items;          // pixel-wise work list (persistent kernels)
+    int pass_blocks;             // blocks of the persistent pass (all forward kernels that run)
     int gw_pixels;
-    const uint32_t *gw_exoff;    // per tile: its later-segment items' offset from num_gauss0
-    float4 *gw_sum;              // per Gaussian-wise item, per pixel: the segment summary
+    const uint2 *gw_ent;         // Gaussian-wise segments (tile, segment)
+    const uint2 *gw_tile;        // per Gaussian-wise tile: (its first segment's entry, its second's)
+    float4 *gw_sum;              // per Gaussian-wise segment, per pixel of a full tile: the summary
+    uint32_t *gw_done;           // per (first segment, block): all pixels stopped in it, outputs written
     unsigned int *tile_cost;     // per tile (nullable, zeroed): the largest n_contrib of its pixels
     int pixel_rows;              // Q of the pixel-wise items
     int chunk;
 };
 
-// A pixel's record of one Gaussian-wise segment (2 x 16 bytes), per (segment item, pixel).
-// Written by the segment item:
+// A pixel's record of one Gaussian-wise segment (2 x 16 bytes), per (segment, pixel of the tile).
+// Written by the segment's item:
 //   cd = colour and depth accumulated with the segment's own transmittance from 1;
 //   t  = (transmittance after the segment, last contributor (index in the tile's list, bits;
 //        -1: none), contributing pairs (bits), entries up to and including the stop (bits)
@@ -343,7 +351,7 @@ struct BwdArgs {
     int chunk;
     // segmented walk of the tiles the last forward split (bseg_mode: its render mode, -1:
     // none): the forward's per-tile segment item positions and boundary states
-    int bseg_mode, heavy_threshold, gw_pixels;
+    int bseg_mode, heavy_threshold;
     const uint2 *gw_tile;
     const GwSum *gw_sum;
 };
@@ -433,20 +441,27 @@ cudaError_t launch_pack(long long N, const float *means2D, const float *conic_op
 // first items and the ctrl counts; k_wl_emit writes the items (positions past `capacity`
 // items raise BGS_CHECK_OVERFLOW and are skipped).  The order of tiles within one key is
 // unspecified.
-// gw_segment: entries per Gaussian-wise segment (0: lists are not split); exoff [num_tiles]
-// (nullable when gw_segment is 0) receives each tile's later-segment offset; extra_cap: the
-// most later-segment items the list may hold (beyond it the lists are not split).
+// gw_segment: entries per Gaussian-wise segment (0: no tile is Gaussian-wise); extra_cap: the
+// most later segments the list may hold (beyond it the lists are not split).
 // bseg_mode >= 0 (a pixel-wise list for the backward): the tiles that the last forward, in
 // that render mode, split into segments get their pixel-wise items once per segment
-// (ctrl->gw_seg, the forward's segment length, is kept).  gw_tile [num_tiles] (nullable):
-// per Gaussian-wise tile of a forward list, (first first-segment item, first later-segment
-// item).  cost [num_tiles] (nullable): the per-tile load that orders the list heaviest first
-// (default: the list length).
+// (ctrl->gw_seg, the forward's segment length, is kept).  gw (null pointers for a list without
+// Gaussian-wise tiles): exoff [num_tiles] scratch, the segments' entries ent [ent_cap], per
+// tile the entries of its first and second segment, and the cleared flags done.  cost
+// [num_tiles] (nullable): the per-tile load that orders the list heaviest first (default: the
+// list length).
+struct GwLists {
+    uint32_t *exoff;
+    uint2 *ent;
+    long long ent_cap;
+    uint2 *tile;
+    uint32_t *done;
+};
 cudaError_t launch_worklist_buckets(const uint2 *ranges, int num_tiles, const ViewTable &vt, int tile_w, int tile_h,
                                     int mode, int heavy_threshold, int lpt, int gw_pixels, int pixel_rows,
-                                    int gw_segment, long long extra_cap, uint32_t *slot, uint32_t *exoff,
-                                    uint2 *items, long long capacity, int bseg_mode, uint2 *gw_tile,
-                                    const uint32_t *cost, DevCtrl *ctrl, cudaStream_t s);
+                                    int gw_segment, long long extra_cap, uint32_t *slot, uint2 *items,
+                                    long long capacity, int bseg_mode, const GwLists &gw, const uint32_t *cost,
+                                    int num_sms, DevCtrl *ctrl, cudaStream_t s);
 
 // queue of the current list: rewind for another pass / mark exhausted (fault injection)
 cudaError_t launch_rewind_queue(DevCtrl *ctrl, cudaStream_t s);
@@ -455,12 +470,11 @@ cudaError_t launch_exhaust_queue(DevCtrl *ctrl, cudaStream_t s);
 cudaError_t launch_forward_static(const FwdArgs &a, cudaStream_t s);
 cudaError_t launch_forward_gauss(const FwdArgs &a, int grid, cudaStream_t s);
 cudaError_t launch_forward_pixel(const FwdArgs &a, int grid, bool after_gauss, cudaStream_t s);
-// composes the Gaussian-wise segment summaries per pixel; after both forward kernels
-cudaError_t launch_forward_gw_merge(const FwdArgs &a, int grid, cudaStream_t s);
+// composes the Gaussian-wise segment summaries per pixel; after the other forward kernels
+cudaError_t launch_forward_gw_merge(const FwdArgs &a, int num_sms, cudaStream_t s);
 int forward_balanced_block_threads();
-const void *forward_gauss_kernel(int gw_pixels);
-const void *forward_gw_merge_kernel(int gw_pixels);
 const void *forward_pixel_kernel(int pixel_rows);
+int forward_gauss_grid(const FwdArgs &a, int num_sms, int max_per_sm);
 
 cudaError_t launch_backward_static(const BwdArgs &a, cudaStream_t s);
 cudaError_t launch_backward_balanced(const BwdArgs &a, int grid, cudaStream_t s);

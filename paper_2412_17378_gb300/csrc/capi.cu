@@ -93,8 +93,9 @@ struct bgs_plan {
     int smem_optin = 0;
     // render
     Buf recs, tile_idx, items, grad_acc, warp_items;  // tile_idx: each tile's slot in its work-list bucket
-    Buf gw_exoff, gw_sum, gw_tile;  // Gaussian-wise segments: per-tile later-segment offsets, per-item
-                                    // summaries, per-tile segment item positions
+    Buf gw_exoff, gw_ent, gw_tile, gw_done, gw_sum;  // Gaussian-wise segments: per-tile later-segment
+                                                     // offsets, entries, per-tile entry numbers, per-block
+                                                     // flags, per-pixel summaries
     Buf tile_cost;                  // per-tile largest n_contrib, from the last forward (the
                                     // backward's work-list order); valid for cost_key's tiles
     // batched binning: depth keys of every view
@@ -280,12 +281,12 @@ long long gw_groups(const bgs_plan *p, int tw, int th) {
     return ((long long)tw * th + p->desc.gw_pixels - 1) / p->desc.gw_pixels;
 }
 
-// Most later-segment items a list over num_entries entries is given: one per (segment after
-// a tile's first, pixel group) when the tile ranges do not overlap, at most 2^24; beyond it
+// Most later segments a list over num_entries entries is given: one per segment after a
+// tile's first when the tile ranges do not overlap, at most 2^24 pixel-group items; beyond it
 // no list is split.
 long long gw_extra_cap(const bgs_plan *p, int tw, int th, int64_t num_entries) {
     const long long L = p->desc.gw_segment;
-    return std::min<long long>(gw_groups(p, tw, th) * (num_entries / L + 1), 1ll << 24);
+    return std::min<long long>(num_entries / L + 1, (1ll << 24) / gw_groups(p, tw, th));
 }
 
 // mode: the render mode; AUTO with a threshold no list can exceed queues every tile
@@ -298,35 +299,39 @@ int build_worklist(bgs_plan *p, const uint32_t *ranges, const bgs::ViewTable &vt
                                   (int64_t)p->desc.heavy_threshold >= num_entries))
         mode = BGS_MODE_PIXEL;
     const int T = vt.tile_base[vt.V];
-    const int P = p->desc.gw_pixels;
     const uint2 *rg = reinterpret_cast<const uint2 *>(ranges);
     const int item_w = bgs::pix_item_w(p->desc.pixel_rows), item_h = bgs::pix_item_h(p->desc.pixel_rows);
-    const long long per_tile = std::max<long long>(((tw + item_w - 1) / item_w) * ((th + item_h - 1) / item_h),
-                                                   (tw * th + P - 1) / P);
     const bool gauss = gauss_possible(p, mode, num_entries);
     const long long extra_cap = gauss ? gw_extra_cap(p, tw, th, num_entries) : 0;
     // a segmented backward list: the tiles' pixel-wise items once per segment, at most as many
     // more segments as the forward's split (which fit its budget) had
     const long long pix_per_tile = ((tw + item_w - 1) / item_w) * ((th + item_h - 1) / item_h);
-    const long long bseg_extra =
-        bseg_mode >= 0 ? pix_per_tile * (gw_extra_cap(p, tw, th, num_entries) / gw_groups(p, tw, th) + 1) : 0;
-    const long long max_items = (long long)T * per_tile + extra_cap + bseg_extra;
+    const long long bseg_extra = bseg_mode >= 0 ? pix_per_tile * (gw_extra_cap(p, tw, th, num_entries) + 1) : 0;
+    const long long pix_items = (long long)T * pix_per_tile + bseg_extra;
+    const long long entries = gauss ? (long long)T + extra_cap : 0;  // Gaussian-wise segments
+    const long long nb = bgs::gw_blocks_per(tw, th);
+    const long long max_items = pix_items + entries * std::max(gw_groups(p, tw, th), nb);
     if (max_items >= (1ll << 31)) return fail(BGS_ERR_INVALID, "too many work items (%lld)", max_items);
     BGS_TRY(ensure(p, p->tile_idx, sizeof(uint32_t) * T, s, "tile_idx"));
-    BGS_TRY(ensure(p, p->items, sizeof(uint2) * max_items, s, "items"));
+    BGS_TRY(ensure(p, p->items, sizeof(uint2) * pix_items, s, "items"));
+    bgs::GwLists gw = {};
     if (gauss) {
         BGS_TRY(ensure(p, p->gw_exoff, sizeof(uint32_t) * T, s, "gw_exoff"));
-        // summaries of the Gaussian-wise items: first segments of at most every tile, plus
-        // the later segments
-        const long long gw_items = (long long)T * gw_groups(p, tw, th) + extra_cap;
-        BGS_TRY(ensure(p, p->gw_sum, (size_t)gw_items * P * 2 * sizeof(float4), s, "gw_sum"));
+        BGS_TRY(ensure(p, p->gw_ent, sizeof(uint2) * entries, s, "gw_ent"));
         BGS_TRY(ensure(p, p->gw_tile, sizeof(uint2) * T, s, "gw_tile"));
+        BGS_TRY(ensure(p, p->gw_done, sizeof(uint32_t) * T * nb, s, "gw_done"));
+        BGS_TRY(ensure(p, p->gw_sum, (size_t)entries * tw * th * sizeof(bgs::GwSum), s, "gw_sum"));
+        gw.exoff = (uint32_t *)p->gw_exoff.p;
+        gw.ent = (uint2 *)p->gw_ent.p;
+        gw.ent_cap = entries;
+        gw.tile = (uint2 *)p->gw_tile.p;
+        gw.done = (uint32_t *)p->gw_done.p;
     }
-    BGS_CUDA(bgs::launch_worklist_buckets(rg, T, vt, tw, th, mode, p->desc.heavy_threshold, p->desc.lpt_order, P,
-                                          p->desc.pixel_rows, gauss ? p->desc.gw_segment : 0, extra_cap,
-                                          (uint32_t *)p->tile_idx.p, gauss ? (uint32_t *)p->gw_exoff.p : nullptr,
-                                          (uint2 *)p->items.p, (long long)(p->items.bytes / sizeof(uint2)), bseg_mode,
-                                          gauss ? (uint2 *)p->gw_tile.p : nullptr, cost, p->ctrl, s),
+    BGS_CUDA(bgs::launch_worklist_buckets(rg, T, vt, tw, th, mode, p->desc.heavy_threshold, p->desc.lpt_order,
+                                          p->desc.gw_pixels, p->desc.pixel_rows, gauss ? p->desc.gw_segment : 0,
+                                          extra_cap, (uint32_t *)p->tile_idx.p, (uint2 *)p->items.p,
+                                          (long long)(p->items.bytes / sizeof(uint2)), bseg_mode, gw, cost,
+                                          p->num_sms, p->ctrl, s),
              "build_worklist");
     p->host_launches += T > 0 ? 2 : 1;
     p->wl_key = worklist_key(p, ranges, vt, tw, th, mode, bseg_mode, cost ? 1 : 0);
@@ -418,7 +423,7 @@ int bgs_plan_destroy(bgs_plan *p) {
         for (Buf *b : sb)
             if (b->p) cudaFree(b->p);
     }
-    Buf *bufs[] = {&p->gw_exoff, &p->gw_sum, &p->gw_tile, &p->tile_cost, &p->vkey_sorted, &p->touched, &p->touched_sorted, &p->dkey,
+    Buf *bufs[] = {&p->gw_exoff, &p->gw_ent, &p->gw_done, &p->gw_sum, &p->gw_tile, &p->tile_cost, &p->vkey_sorted, &p->touched, &p->touched_sorted, &p->dkey,
                    &p->dkey_sorted, &p->gidx, &p->order, &p->offsets,
                    &p->keys_in, &p->keys_out, &p->vals_in, &p->cub_tmp, &p->recs,
                    &p->tile_idx, &p->items, &p->warp_items,
@@ -495,11 +500,10 @@ size_t bgs_workspace_size(const bgs_plan *p, int64_t N, int64_t K, int64_t T, in
     s += 8 * K * 2 + 4 * K;             // keys in/out, values in
     s += 48 * N * 2;                    // packed records, gradient accumulators
     s += 4 * T;                         // work-list bucket slots
-    s += 8 * T * (size_t)std::max(8, (256 + P - 1) / P);  // work items (16x16 tiles)
+    s += 8 * T * 8;                     // work items (16x16 tiles)
     if ((int64_t)p->desc.heavy_threshold < K) {  // Gaussian-wise segments (AUTO)
-        const size_t groups = (256 + P - 1) / P;
-        const size_t extra = std::min<size_t>(groups * ((size_t)K / p->desc.gw_segment + 1), (size_t)1 << 24);
-        s += 8 * extra + 4 * T + (groups * T + extra) * P * 32;
+        const size_t entries = T + std::min<size_t>((size_t)K / p->desc.gw_segment + 1, ((size_t)1 << 24) / (256 / P));
+        s += entries * (8 + 256 * 32) + T * (4 + 8 + 16);
     }
     s += 64 << 20;                      // CUB temporaries (upper estimate)
     return s;
@@ -557,16 +561,17 @@ int bgs_plan_reserve(bgs_plan *p, int64_t N, int64_t K, int64_t T, int64_t pixel
     BGS_TRY(ensure(p, p->vals_in, 4 * K, s, "vals_in"));
     BGS_TRY(ensure(p, p->recs, sizeof(bgs::Rec) * N, s, "recs"));
     BGS_TRY(ensure(p, p->grad_acc, sizeof(bgs::Rec) * N, s, "grad_acc"));
-    const int P = p->desc.gw_pixels;
     BGS_TRY(ensure(p, p->tile_idx, 4 * T, s, "per-tile"));
-    // work items (16 x 16 tiles); with Gaussian-wise items possible in AUTO mode, the segment
-    // items and summaries too
-    const bool gauss = (int64_t)p->desc.heavy_threshold < K;
-    const long long extra = gauss ? gw_extra_cap(p, 16, 16, K) : 0;
-    BGS_TRY(ensure(p, p->items, 8 * (T * (size_t)std::max(8, (256 + P - 1) / P) + (size_t)extra), s, "items"));
-    if (gauss) {
+    // work items (16 x 16 tiles); with Gaussian-wise tiles possible in AUTO mode, the segments'
+    // entries and summaries too
+    BGS_TRY(ensure(p, p->items, 8 * T * (size_t)8, s, "items"));
+    if ((int64_t)p->desc.heavy_threshold < K) {
+        const size_t entries = (size_t)T + (size_t)gw_extra_cap(p, 16, 16, K);
         BGS_TRY(ensure(p, p->gw_exoff, 4 * T, s, "gw_exoff"));
-        BGS_TRY(ensure(p, p->gw_sum, ((size_t)T * gw_groups(p, 16, 16) + (size_t)extra) * P * 32, s, "gw_sum"));
+        BGS_TRY(ensure(p, p->gw_ent, 8 * entries, s, "gw_ent"));
+        BGS_TRY(ensure(p, p->gw_tile, 8 * T, s, "gw_tile"));
+        BGS_TRY(ensure(p, p->gw_done, 4 * T * (size_t)bgs::gw_blocks_per(16, 16), s, "gw_done"));
+        BGS_TRY(ensure(p, p->gw_sum, entries * 256 * sizeof(bgs::GwSum), s, "gw_sum"));
     }
     // CUB temporaries: the largest of the depth sort, the N-scan, the tile sort and the tile scan
     size_t t[4] = {0, 0, 0, 0};
@@ -980,12 +985,17 @@ int render_forward_impl(bgs_plan *p, const bgs::ViewTable &vt, const bgs::ViewOu
     BGS_TRY(build_worklist(p, ranges, vt, tw, th, mode, num_entries, s));
     a.items = (const uint2 *)p->items.p;
     const int threads = bgs::forward_balanced_block_threads();
-    const int grid_g = grid_for(p, bgs::forward_gauss_kernel(a.gw_pixels), threads);
     const int grid_p = grid_for(p, bgs::forward_pixel_kernel(a.pixel_rows), threads);
     // AUTO with a threshold no list can exceed queues no Gaussian-wise item
     const bool gauss = gauss_possible(p, mode, num_entries);
-    a.gw_exoff = gauss ? (const uint32_t *)p->gw_exoff.p : nullptr;
-    a.gw_sum = gauss ? (float4 *)p->gw_sum.p : nullptr;
+    int grid_g = 0;
+    if (gauss) {
+        a.gw_ent = (const uint2 *)p->gw_ent.p;
+        a.gw_tile = (const uint2 *)p->gw_tile.p;
+        a.gw_done = (uint32_t *)p->gw_done.p;
+        a.gw_sum = (float4 *)p->gw_sum.p;
+        grid_g = bgs::forward_gauss_grid(a, p->num_sms, p->desc.blocks_per_sm);
+    }
     {  // the backward's per-tile cost, gathered by the forward kernels
         const int T = vt.tile_base[vt.V];
         BGS_TRY(ensure(p, p->tile_cost, sizeof(uint32_t) * std::max(T, 1), s, "tile_cost"));
@@ -994,17 +1004,16 @@ int render_forward_impl(bgs_plan *p, const bgs::ViewTable &vt, const bgs::ViewOu
         p->cost_key = worklist_key(p, ranges, vt, tw, th, BGS_MODE_PIXEL);
         p->cost_valid = true;
     }
-    a.pass_blocks = (gauss ? grid_g : 0) + (mode != BGS_MODE_GAUSSIAN ? grid_p : 0);
+    a.pass_blocks = grid_g + (mode != BGS_MODE_GAUSSIAN ? grid_p : 0);
     BGS_TRY(inject_pending_fault(p, s));
     KernelTimer kt(p, s, &p->ev_fwd);
     if (gauss) BGS_CUDA(bgs::launch_forward_gauss(a, grid_g, s), "forward_gauss");
     if (mode != BGS_MODE_GAUSSIAN) BGS_CUDA(bgs::launch_forward_pixel(a, grid_p, gauss, s), "forward_pixel");
-    if (gauss) BGS_CUDA(bgs::launch_forward_gw_merge(a, grid_for(p, bgs::forward_gw_merge_kernel(a.gw_pixels), threads), s),
-                        "forward_gw_merge");
+    if (gauss) BGS_CUDA(bgs::launch_forward_gw_merge(a, p->num_sms, s), "forward_gw_merge");
     p->gw_fwd_valid = gauss;
     p->gw_fwd_key = p->wl_key;
     kt.stop();
-    p->host_launches += (gauss && mode != BGS_MODE_GAUSSIAN) ? 3 : (gauss ? 2 : 1);
+    p->host_launches += (gauss ? 2 : 0) + (mode != BGS_MODE_GAUSSIAN ? 1 : 0);
     return BGS_OK;
 }
 
@@ -1065,7 +1074,6 @@ int render_backward_impl(bgs_plan *p, const bgs::ViewTable &vt, const bgs::ViewG
         const int bseg = (p->gw_fwd_valid && memcmp(&fk, &p->gw_fwd_key, sizeof fk) == 0) ? mode : -1;
         a.bseg_mode = bseg;
         a.heavy_threshold = p->desc.heavy_threshold;
-        a.gw_pixels = p->desc.gw_pixels;
         a.gw_tile = bseg >= 0 ? (const uint2 *)p->gw_tile.p : nullptr;
         a.gw_sum = bseg >= 0 ? (const bgs::GwSum *)p->gw_sum.p : nullptr;
         // heaviest first by what the backward walks: each tile's largest n_contrib, which the

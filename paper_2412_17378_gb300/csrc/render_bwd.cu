@@ -385,11 +385,9 @@ __device__ __forceinline__ PixState enter_pixel(const BwdArgs &a, const ItemGeom
             t.nc = 0;  // nothing of this pixel in the segment
         } else if (end >= g.e1 && inside) {
             // enter from behind: the merge's state at the segment's end
-            const int P = a.gw_pixels, groups = (g.vw * g.vh + P - 1) / P;
-            const int qp = (py - g.y0) * g.vw + (px - g.x0), group = qp / P;
             const uint2 gt = a.gw_tile[g.tile];
-            const size_t si = g.seg == 0 ? (size_t)gt.x + group : (size_t)gt.y + (size_t)(g.seg - 1) * groups + group;
-            const GwSum st = a.gw_sum[si * P + qp % P];
+            const size_t entry = g.seg == 0 ? (size_t)gt.x : (size_t)gt.y + (size_t)(g.seg - 1);
+            const GwSum st = a.gw_sum[entry * (size_t)(a.tile_w * a.tile_h) + (py - g.y0) * g.vw + (px - g.x0)];
             const float iT = 1.f / st.t.x;
             t.T = st.t.x;
             t.Rg = (st.cd.x * t.g0 + st.cd.y * t.g1 + st.cd.z * t.g2) * iT;
@@ -557,7 +555,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (Q <= 4 && !Extra) ? 4 : (Q <=
         const unsigned end = min(first + chunk, num_items);
         for (unsigned it = first; it < end; ++it) {
             const uint2 item = a.items[it];
-            const ItemGeom ig = item_geom<Q>(a, (int)item.x, (int)(item.y & ~kKindGauss), L);
+            const ItemGeom ig = item_geom<Q>(a, (int)item.x, (int)item.y, L);
             if (!bwd_pixel_item<Q, Extra>(a, ig, buf, lane)) bwd_pixel_item_wild<Q, Extra>(a, ig, lane);
             ++st_items;
         }

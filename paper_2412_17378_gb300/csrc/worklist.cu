@@ -5,12 +5,14 @@
 // between the Gaussian-wise and the pixel-wise kernel.  Here the choice is made per
 // tile from its list length n (the paper names "the Gaussians of a tile" as the key
 // load-balance metric, Sec. 4.4):
-//   n >  heavy_threshold -> Gaussian-wise items of P pixels (one warp each), and, for a list
-//                           longer than gw_segment entries, one item per further segment
-//                           of gw_segment entries and P pixels (the cross-warp split),
+//   n >  heavy_threshold -> Gaussian-wise: one segment entry, and, for a list longer than
+//                           gw_segment entries, one per further segment of gw_segment
+//                           entries (the cross-warp split),
 //   n <= heavy_threshold -> pixel-wise items of 8 x 4Q pixels (one warp, Q pixels per lane).
-// The work list holds the Gaussian-wise first-segment items, then the later-segment items,
-// then the pixel-wise items.
+// The segment list holds the tiles' first segments, then the later ones.  Each entry stands for
+// a fixed number of items, one warp each: the tile's 8 x 8 blocks of pixels (two to a lane) or
+// its groups of P pixels (the lanes splitting the entries).  Item numbers count the segments'
+// items first, then the pixel-wise ones.
 // Tiles of all views of a batched call share one global tile space.
 // Items of heavier tiles are queued first (longest-processing-time order) so the long
 // items start early and the light ones fill the tail.
@@ -20,15 +22,12 @@
 
 namespace bgs {
 
-// Items of tile t: Gaussian-wise (first segments), P pixels each; else pixel-wise sub-blocks of
-// its visible part.
-__device__ __forceinline__ uint32_t tile_items(int t, bool gauss, const ViewTable &vt, int tile_w, int tile_h,
-                                               int gw_pixels, int pixel_rows) {
+// Pixel-wise items of tile t: the sub-blocks of its visible part.
+__device__ __forceinline__ uint32_t tile_items(int t, const ViewTable &vt, int tile_w, int tile_h, int pixel_rows) {
     const int v = view_of(vt, t);
     const int lt = t - vt.tile_base[v];
     const int tx = lt % vt.tiles_x[v], ty = lt / vt.tiles_x[v];
     const int vw = min(tile_w, vt.W[v] - tx * tile_w), vh = min(tile_h, vt.H[v] - ty * tile_h);
-    if (gauss) return (uint32_t)((vw * vh + gw_pixels - 1) / gw_pixels);
     const int iw = pix_item_w(pixel_rows), ih = pix_item_h(pixel_rows);
     return (uint32_t)(((vw + iw - 1) / iw) * ((vh + ih - 1) / ih));
 }
@@ -42,12 +41,17 @@ __device__ __forceinline__ uint32_t bwd_segments(int bseg_mode, int heavy_thresh
     return (n - 1u) / L + 1u;
 }
 
-// Later-segment items of a Gaussian-wise tile with first-segment items `groups` and list
-// length n: one per (segment after the first, pixel group).
-__device__ __forceinline__ unsigned long long tile_extra(bool gauss, uint32_t groups, uint32_t n, int gw_segment) {
-    if (!gauss || gw_segment <= 0 || n <= (uint32_t)gw_segment) return 0ull;
-    return (unsigned long long)groups * (unsigned long long)((n - 1u) / (uint32_t)gw_segment);
+// Segments after the first of a tile with list length n.
+__device__ __forceinline__ uint32_t tile_extra(bool gauss, uint32_t n, int gw_segment) {
+    return !gauss || gw_segment <= 0 || n <= (uint32_t)gw_segment ? 0u : (n - 1u) / (uint32_t)gw_segment;
 }
+
+// Where the segments alone give every SM at least this many blocks of pixels, their items are
+// those blocks, which do a fifth of the work; below, a few warps would walk long segments one
+// record after the other while the chip idles, and the items are pixel groups, 16 times as many
+// at 4 pixels (a 256 x 256 frame of 10k Gaussians, 30 tiles past the threshold: 275 us with
+// groups, 382 with blocks).
+constexpr unsigned int kWideBlocksPerSm = 2;
 
 // The list is ordered by a descending 8-bit key per tile: its kind in the top bit (Gaussian-
 // wise tiles first) and, when lpt is on, a log-scale bucket of its list length below it
@@ -74,18 +78,19 @@ __device__ __forceinline__ uint32_t wl_sort_key(uint32_t n, bool gauss, int lpt)
 }
 
 // Per block: items per key in shared memory (a tile's slot within its block's share is the
-// atomic's old value), then one global atomic per key gives the block's share its place in
-// the key's bucket; a block scan of the tiles' later-segment items and one global atomic
-// give each tile its later-segment offset.  The last block to finish reads the totals
-// (clearing them for the next build), scans them in descending key order into the buckets'
-// first items and publishes the list's item counts and queue cursors.  When the
-// later-segment items exceed extra_cap, no list is split (segment size 0).
+// atomic's old value; a Gaussian-wise tile counts one), then one global atomic per key gives
+// the block's share its place in the key's bucket; a block scan of the tiles' later segments
+// and one global atomic give each tile its later-segment offset.  The last block to finish
+// reads the totals (clearing them for the next build), scans them in descending key order into
+// the buckets' first items and publishes the list's item counts and queue cursors.  When the
+// later segments exceed extra_cap, no list is split (segment size 0).
 __global__ void __launch_bounds__(kWlcThreads) k_wl_count(const uint2 *__restrict__ ranges, int T, const ViewTable vt,
                                                            int tile_w, int tile_h, int mode, int heavy_threshold,
                                                            int lpt, int gw_pixels, int pixel_rows, int gw_segment,
                                                            long long extra_cap, uint32_t *__restrict__ slot,
                                                            uint32_t *__restrict__ exoff, int bseg_mode,
-                                                           const uint32_t *__restrict__ cost, DevCtrl *ctrl) {
+                                                           const uint32_t *__restrict__ cost, int num_sms,
+                                                           DevCtrl *ctrl) {
     using Scan = cub::BlockScan<uint32_t, kWlcThreads>;
     using Scan64 = cub::BlockScan<unsigned long long, kWlcThreads>;
     __shared__ union {
@@ -95,6 +100,7 @@ __global__ void __launch_bounds__(kWlcThreads) k_wl_count(const uint2 *__restric
     __shared__ uint32_t s_cnt[256], s_base[256];
     __shared__ unsigned long long s_xbase;
     __shared__ bool s_last;
+    __shared__ uint32_t s_first;
     s_cnt[threadIdx.x] = 0u;
     __syncthreads();
     const int t = blockIdx.x * kWlcThreads + threadIdx.x;
@@ -107,10 +113,11 @@ __global__ void __launch_bounds__(kWlcThreads) k_wl_count(const uint2 *__restric
         const uint32_t n = rg.y >= rg.x ? rg.y - rg.x : 0u;
         const bool gauss = tile_is_gauss(mode, heavy_threshold, n);
         key = wl_sort_key(cost ? cost[t] : n, gauss, lpt);
-        const uint32_t c = tile_items(t, gauss, vt, tile_w, tile_h, gw_pixels, pixel_rows) *
-                           (gauss ? 1u : bwd_segments(bseg_mode, heavy_threshold, Lb, n));
+        const uint32_t c = gauss ? 1u
+                                 : tile_items(t, vt, tile_w, tile_h, pixel_rows) *
+                                       bwd_segments(bseg_mode, heavy_threshold, Lb, n);
         local = atomicAdd(&s_cnt[key], c);
-        extra = tile_extra(gauss, c, n, gw_segment);
+        extra = tile_extra(gauss, n, gw_segment);
     }
     if (gw_segment > 0) {  // grid-uniform
         unsigned long long xoff, xtotal;
@@ -146,18 +153,23 @@ __global__ void __launch_bounds__(kWlcThreads) k_wl_count(const uint2 *__restric
     const uint32_t c = atomicExch(&ctrl->wl_cnt[k], 0u);
     uint32_t off, total;
     Scan(scan_tmp.s32).ExclusiveSum(c, off, total);
-    // Gaussian-wise keys (kind bit set) are the largest; the pixel-wise buckets follow the
-    // later-segment items, and the first pixel-wise key's offset is the number of
-    // first-segment items
+    // Gaussian-wise keys (kind bit set) are the largest: the first pixel-wise key's offset is
+    // the number of first segments
     const int pix_top = lpt ? 127 : 0;
-    ctrl->wl_off[k] = k <= pix_top ? off + E : off;
-    if (k == pix_top) {
-        ctrl->num_gauss0 = off;
-        ctrl->num_gauss = off + E;
-        ctrl->queue_head = off + E;
-    }
+    if (k == pix_top) s_first = off;
+    __syncthreads();
+    const uint32_t first = s_first;
+    ctrl->wl_off[k] = k <= pix_top ? off - first : off;
     if (threadIdx.x == 0) {
-        ctrl->num_items = total + E;
+        const unsigned long long blocks = (unsigned long long)(first + E) * gw_blocks_per(tile_w, tile_h);
+        const bool wide = blocks >= (unsigned long long)kWideBlocksPerSm * num_sms;
+        const uint32_t G = (first + E) * (wide ? gw_blocks_per(tile_w, tile_h)
+                                               : (tile_w * tile_h + gw_pixels - 1) / gw_pixels);
+        ctrl->gw_wide = wide ? 1u : 0u;
+        ctrl->gw_first = first;
+        ctrl->num_gauss = G;
+        ctrl->queue_head = G;
+        ctrl->num_items = G + total - first;
         ctrl->queue_head_g = 0u;
         ctrl->pass_items = 0u;
         ctrl->warps_done = 0u;
@@ -165,58 +177,57 @@ __global__ void __launch_bounds__(kWlcThreads) k_wl_count(const uint2 *__restric
     }
 }
 
-// A thread per tile writes the tile's items at its bucket's first item + its slot, and its
-// later-segment items (sub-item index = segment * groups + group, segment >= 1) at
-// num_gauss0 + its offset.
+// A thread per tile writes the tile's pixel-wise items at its bucket's first item + its slot,
+// or its segment entries: the first at that place of the first segments, the later ones at
+// gw_first + its offset.
 __global__ void __launch_bounds__(256) k_wl_emit(const uint2 *__restrict__ ranges, int T, const ViewTable vt,
                                                  int tile_w, int tile_h, int mode, int heavy_threshold, int lpt,
-                                                 int gw_pixels, int pixel_rows, const uint32_t *__restrict__ slot,
-                                                 const uint32_t *__restrict__ exoff, uint2 *__restrict__ items,
-                                                 long long capacity, int bseg_mode, uint2 *__restrict__ gw_tile,
-                                                 const uint32_t *__restrict__ cost, DevCtrl *ctrl) {
+                                                 int pixel_rows, const uint32_t *__restrict__ slot,
+                                                 uint2 *__restrict__ items, long long capacity, int bseg_mode,
+                                                 const GwLists gw, const uint32_t *__restrict__ cost, DevCtrl *ctrl) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     const uint2 rg = ranges[t];
     const uint32_t n = rg.y >= rg.x ? rg.y - rg.x : 0u;
     const bool gauss = tile_is_gauss(mode, heavy_threshold, n);
-    const unsigned Lb = bseg_mode >= 0 ? ctrl->gw_seg : 0u;
-    const uint32_t c = tile_items(t, gauss, vt, tile_w, tile_h, gw_pixels, pixel_rows) *
-                       (gauss ? 1u : bwd_segments(bseg_mode, heavy_threshold, Lb, n));
     const long long pos = (long long)ctrl->wl_off[wl_sort_key(cost ? cost[t] : n, gauss, lpt)] + slot[t];
+    if (gauss) {
+        const uint32_t x = tile_extra(true, n, (int)ctrl->gw_seg);
+        const long long xpos = (long long)ctrl->gw_first + (x ? gw.exoff[t] : 0u);
+        if (pos >= gw.ent_cap || xpos + x > gw.ent_cap) {
+            raise_check(ctrl, BGS_CHECK_OVERFLOW);
+            return;
+        }
+        gw.ent[pos] = make_uint2((uint32_t)t, 0u);
+        for (uint32_t q = 0; q < x; ++q) gw.ent[xpos + q] = make_uint2((uint32_t)t, q + 1u);
+        gw.tile[t] = make_uint2((uint32_t)pos, (uint32_t)xpos);
+        const int nb = gw_blocks_per(tile_w, tile_h);
+        for (int q = 0; q < nb; ++q) gw.done[pos * nb + q] = 0u;
+        return;
+    }
+    const unsigned Lb = bseg_mode >= 0 ? ctrl->gw_seg : 0u;
+    const uint32_t c = tile_items(t, vt, tile_w, tile_h, pixel_rows) * bwd_segments(bseg_mode, heavy_threshold, Lb, n);
     if (pos + (long long)c > capacity) {
         raise_check(ctrl, BGS_CHECK_OVERFLOW);
         return;
     }
-    const uint32_t kindbit = gauss ? kKindGauss : 0u;
-    for (uint32_t q = 0; q < c; ++q) items[pos + q] = make_uint2((uint32_t)t, kindbit | q);
-    const int seg = (int)ctrl->gw_seg;
-    const unsigned long long x = tile_extra(gauss, c, n, seg);
-    // where a Gaussian-wise tile's segment items sit (for a backward that reads their summaries)
-    if (gw_tile && gauss) gw_tile[t] = make_uint2((uint32_t)pos, x ? ctrl->num_gauss0 + exoff[t] : 0u);
-    if (x == 0ull) return;
-    const long long xpos = (long long)ctrl->num_gauss0 + exoff[t];
-    if (xpos + (long long)x > capacity) {
-        raise_check(ctrl, BGS_CHECK_OVERFLOW);
-        return;
-    }
-    for (uint32_t q = 0; q < (uint32_t)x; ++q) items[xpos + q] = make_uint2((uint32_t)t, kKindGauss | (c + q));
+    for (uint32_t q = 0; q < c; ++q) items[pos + q] = make_uint2((uint32_t)t, q);
 }
 
 cudaError_t launch_worklist_buckets(const uint2 *ranges, int num_tiles, const ViewTable &vt, int tile_w, int tile_h,
                                     int mode, int heavy_threshold, int lpt, int gw_pixels, int pixel_rows,
-                                    int gw_segment, long long extra_cap, uint32_t *slot, uint32_t *exoff,
-                                    uint2 *items, long long capacity, int bseg_mode, uint2 *gw_tile,
-                                    const uint32_t *cost, DevCtrl *ctrl, cudaStream_t s) {
-    if (num_tiles < 0 || (gw_segment > 0 && !exoff)) return cudaErrorInvalidValue;
+                                    int gw_segment, long long extra_cap, uint32_t *slot, uint2 *items,
+                                    long long capacity, int bseg_mode, const GwLists &gw, const uint32_t *cost,
+                                    int num_sms, DevCtrl *ctrl, cudaStream_t s) {
+    if (num_tiles < 0 || (gw_segment > 0 && !(gw.exoff && gw.ent && gw.tile && gw.done))) return cudaErrorInvalidValue;
     const int blocks = num_tiles > 0 ? (num_tiles + kWlcThreads - 1) / kWlcThreads : 1;
     k_wl_count<<<blocks, kWlcThreads, 0, s>>>(ranges, num_tiles, vt, tile_w, tile_h, mode, heavy_threshold, lpt,
-                                              gw_pixels, pixel_rows, gw_segment, extra_cap, slot, exoff, bseg_mode,
-                                              cost, ctrl);
+                                              gw_pixels, pixel_rows, gw_segment, extra_cap, slot, gw.exoff, bseg_mode,
+                                              cost, num_sms, ctrl);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || num_tiles == 0) return e;
     k_wl_emit<<<(num_tiles + 255) / 256, 256, 0, s>>>(ranges, num_tiles, vt, tile_w, tile_h, mode, heavy_threshold,
-                                                      lpt, gw_pixels, pixel_rows, slot, exoff, items, capacity,
-                                                      bseg_mode, gw_tile, cost, ctrl);
+                                                      lpt, pixel_rows, slot, items, capacity, bseg_mode, gw, cost, ctrl);
     return cudaGetLastError();
 }
 
