@@ -1,8 +1,10 @@
 // preprocess.cu -- a1: per-Gaussian projection (Eq. 1-3 of the paper, Sec. 2.1).
 //
-// One thread per Gaussian.  The work is ~80 bytes of HBM traffic and ~150 FP32
-// operations per Gaussian: a few microseconds per million Gaussians, far below the
-// render kernels, so the kernel is written for clarity with coalesced scalar loads.
+// One thread per Gaussian over the views, coalesced scalar loads and stores.  With several views
+// both kernels are bound by issue, not by their 36 (28) bytes per record: the forward takes 72
+// us for 1M Gaussians in 8 views (332 MB, 4.4 TB/s; 86 us while every record divided by the
+// tile sides and formed 64-bit indices), the backward 72 us for 4 views (109 us at 16 warps an SM
+// while each view waited for its own loads and chained its own quaternion gradient).
 #include "bgs_internal.cuh"
 
 namespace bgs {
@@ -10,8 +12,12 @@ namespace bgs {
 struct CamDev {
     float V[12];  // rows 0..2 of the world->camera matrix
     float fx, fy, cx, cy, near_plane, lowpass, lim_x, lim_y;
+    float inv_tw, inv_th;  // a tile side's exact reciprocal where it is a power of two, else 0
     int W, H, tile_w, tile_h, tiles_x, tiles_y;
 };
+
+// The exact reciprocal of a power of two (a product by it is the quotient), 0 for another side.
+__host__ __device__ __forceinline__ float tile_recip(int t) { return (t & (t - 1)) == 0 ? 1.f / (float)t : 0.f; }
 
 struct CamTable {
     int V;
@@ -21,17 +27,18 @@ struct CamTable {
 // Tile rectangle of a Gaussian: x in [floor((u-r)/tw), floor((u+(r+tw-1))/tw)), clamped.
 // Float32 with one IEEE rounding per operation (no contraction), the same operations the
 // binning kernel and the host-side checks use.
-// For a power-of-two tile side the quotient is the product by its exact reciprocal.
-__device__ __forceinline__ float tile_quot(float a, int t) {
-    return (t & (t - 1)) == 0 ? __fmul_rn(a, 1.f / (float)t) : __fdiv_rn(a, (float)t);
+// For a power-of-two tile side the quotient is the product by its exact reciprocal inv
+// (tile_recip; 0: another side).
+__device__ __forceinline__ float tile_quot(float a, int t, float inv) {
+    return inv != 0.f ? __fmul_rn(a, inv) : __fdiv_rn(a, (float)t);
 }
 
-__device__ __forceinline__ void tile_rect(float u, float v, int r, int tw, int th, int tx, int ty, int &x0,
-                                          int &x1, int &y0, int &y1) {
-    x0 = (int)floorf(tile_quot(__fsub_rn(u, (float)r), tw));
-    x1 = (int)floorf(tile_quot(__fadd_rn(u, (float)(r + tw - 1)), tw));
-    y0 = (int)floorf(tile_quot(__fsub_rn(v, (float)r), th));
-    y1 = (int)floorf(tile_quot(__fadd_rn(v, (float)(r + th - 1)), th));
+__device__ __forceinline__ void tile_rect(float u, float v, int r, int tw, int th, float inv_tw, float inv_th, int tx,
+                                          int ty, int &x0, int &x1, int &y0, int &y1) {
+    x0 = (int)floorf(tile_quot(__fsub_rn(u, (float)r), tw, inv_tw));
+    x1 = (int)floorf(tile_quot(__fadd_rn(u, (float)(r + tw - 1)), tw, inv_tw));
+    y0 = (int)floorf(tile_quot(__fsub_rn(v, (float)r), th, inv_th));
+    y1 = (int)floorf(tile_quot(__fadd_rn(v, (float)(r + th - 1)), th, inv_th));
     x0 = min(max(x0, 0), tx);
     x1 = min(max(x1, 0), tx);
     y0 = min(max(y0, 0), ty);
@@ -139,7 +146,7 @@ __device__ __forceinline__ bool project(const CamDev &cam, float px, float py, f
 // A thread per Gaussian, over the views: the Gaussian's parameters are read from DRAM once
 // (the views' later reads hit L1), and record v N + g of every view is written (coalesced
 // per view).
-__global__ void __launch_bounds__(256) k_preprocess(long long N, const float *__restrict__ means3D,
+__global__ void __launch_bounds__(128) k_preprocess(long long N, const float *__restrict__ means3D,
                                                     const float *__restrict__ log_scales,
                                                     const float *__restrict__ quats,
                                                     const float *__restrict__ opacities, const CamTable ct,
@@ -152,8 +159,8 @@ __global__ void __launch_bounds__(256) k_preprocess(long long N, const float *__
     const float px = means3D[3 * g], py = means3D[3 * g + 1], pz = means3D[3 * g + 2];
     Proj frame;
     gauss_frame(log_scales, quats, g, frame);
-    for (int view = 0; view < ct.V; ++view) {
-        const long long rec = (long long)view * N + g;
+    uint32_t rec = (uint32_t)g;  // V N < 2^32
+    for (int view = 0; view < ct.V; ++view, rec += (uint32_t)N) {
         const CamDev &cam = ct.cam[view];
         Proj o = frame;
         const bool ok = project(cam, px, py, pz, o);
@@ -173,8 +180,9 @@ __global__ void __launch_bounds__(256) k_preprocess(long long N, const float *__
             m2 = make_float2(u, v);
             co = make_float4(o.c11 * idet, -o.c01 * idet, o.c00 * idet, op);
             int x0, x1, y0, y1;
-            tile_rect(u, v, r, cam.tile_w, cam.tile_h, cam.tiles_x, cam.tiles_y, x0, x1, y0, y1);
-            const long long area = (long long)(x1 - x0) * (long long)(y1 - y0);
+            tile_rect(u, v, r, cam.tile_w, cam.tile_h, cam.inv_tw, cam.inv_th, cam.tiles_x, cam.tiles_y, x0, x1, y0,
+                      y1);
+            const int area = (x1 - x0) * (y1 - y0);  // fewer tiles than pixels / 32
             if (area > 0) {
                 radius = r;
                 touched = (uint32_t)area;
@@ -196,7 +204,7 @@ __global__ void __launch_bounds__(256) k_preprocess(long long N, const float *__
 //   means2D = (fx x / z + cx, fy y / z + cy), depth = z, t = W p + w;
 //   Sigma = M M^T, M = R S: dL/dM = 2 dL/dSigma M, dL/dlog s_k = s_k sum_r dL/dM_rk R_rk,
 //   dL/dR = dL/dM S, then R(q) and the Jacobian of q / |q|.
-__global__ void __launch_bounds__(256) k_preprocess_backward(long long N, const float *__restrict__ means3D,
+__global__ void __launch_bounds__(128, 5) k_preprocess_backward(long long N, const float *__restrict__ means3D,
                                                              const float *__restrict__ log_scales,
                                                              const float *__restrict__ quats, const CamTable ct,
                                                              const int *__restrict__ radii,
@@ -208,23 +216,46 @@ __global__ void __launch_bounds__(256) k_preprocess_backward(long long N, const 
                                                              float *__restrict__ dL_dquats) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= N) return;
-    float gp[3] = {0.f, 0.f, 0.f}, gls[3] = {0.f, 0.f, 0.f}, gq[4] = {0.f, 0.f, 0.f, 0.f};
+    // summed over the views; gls and gR (dL/dR) still without their factors 2 s_k^2, which like
+    // the chain from R to the quaternion are the same for every view
+    float gp[3] = {0.f, 0.f, 0.f}, gls[3] = {0.f, 0.f, 0.f}, gR[3][3] = {};
+    bool seen = false;
     const float px = means3D[3 * g], py = means3D[3 * g + 1], pz = means3D[3 * g + 2];
     Proj frame;
     gauss_frame(log_scales, quats, g, frame);
+    // A record's radius and incoming gradients are loaded one view ahead: the arithmetic of a
+    // view (about 400 instructions at 16 warps an SM) covers the next one's reads.
+    struct In {
+        int r;
+        float2 m;
+        float a, b, c, d;
+    } next;
+    uint32_t rec = (uint32_t)g;  // V N < 2^32
+    auto load = [&](uint32_t k) {
+        In i;
+        i.r = radii[k];
+        i.m = dL_dmeans2D[k];
+        i.a = dL_dconic[3ull * k], i.b = dL_dconic[3ull * k + 1], i.c = dL_dconic[3ull * k + 2];
+        i.d = dL_ddepths ? dL_ddepths[k] : 0.f;
+        return i;
+    };
+    next = load(rec);
     for (int view = 0; view < ct.V; ++view) {
-        const long long rec = (long long)view * N + g;
-        if (radii[rec] <= 0) continue;
+        const In in = next;
+        rec += (uint32_t)N;
+        if (view + 1 < ct.V) next = load(rec);
+        if (in.r <= 0) continue;
         const CamDev &cam = ct.cam[view];
         Proj o = frame;
         if (!project(cam, px, py, pz, o)) continue;
+        seen = true;
         const float *V = cam.V;
-        const float2 gm = dL_dmeans2D[rec];
-        const float ga = dL_dconic[3 * rec], gb = dL_dconic[3 * rec + 1], gc = dL_dconic[3 * rec + 2];
+        const float2 gm = in.m;
+        const float ga = in.a, gb = in.b, gc = in.c;
         const float iz2 = o.iz * o.iz;
         // means2D and depth
         float gtx = gm.x * cam.fx * o.iz, gty = gm.y * cam.fy * o.iz;
-        float gtz = (dL_ddepths ? dL_ddepths[rec] : 0.f) - (gm.x * cam.fx * o.tx + gm.y * cam.fy * o.ty) * iz2;
+        float gtz = in.d - (gm.x * cam.fx * o.tx + gm.y * cam.fy * o.ty) * iz2;
         // conic -> G = dL/dC2
         const float A = o.c00, B = o.c01, C = o.c11;
         const float idet = 1.f / o.det, id2 = idet * idet;
@@ -269,31 +300,41 @@ __global__ void __launch_bounds__(256) k_preprocess_backward(long long N, const 
 #pragma unroll
         for (int k = 0; k < 3; ++k) gp[k] += V[k] * gtx + V[4 + k] * gty + V[8 + k] * gtz;
         // Sigma = M M^T, M = R S
-        float gR[3][3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const float g0 = dA * Q[0][k] + hB * Q[1][k], g1 = hB * Q[0][k] + dC * Q[1][k];  // G q_k
-            const float s2 = 2.f * o.s[k] * o.s[k];
-            gls[k] += s2 * (Q[0][k] * g0 + Q[1][k] * g1);
+            gls[k] += Q[0][k] * g0 + Q[1][k] * g1;
 #pragma unroll
-            for (int r = 0; r < 3; ++r) gR[r][k] = s2 * (T[0][r] * g0 + T[1][r] * g1);
+            for (int r = 0; r < 3; ++r) gR[r][k] += T[0][r] * g0 + T[1][r] * g1;
         }
-        // R(q) of the normalised quaternion, then d(q / |q|)
-        const float w = o.qw, x = o.qx, y = o.qy, z = o.qz;
-        float dq[4];
-        dq[0] = 2.f * (-z * gR[0][1] + y * gR[0][2] + z * gR[1][0] - x * gR[1][2] - y * gR[2][0] + x * gR[2][1]);
-        dq[1] = 2.f * (y * gR[0][1] + z * gR[0][2] + y * gR[1][0] - 2.f * x * gR[1][1] - w * gR[1][2] + z * gR[2][0] +
-                       w * gR[2][1] - 2.f * x * gR[2][2]);
-        dq[2] = 2.f * (-2.f * y * gR[0][0] + x * gR[0][1] + w * gR[0][2] + x * gR[1][0] + z * gR[1][2] -
-                       w * gR[2][0] + z * gR[2][1] - 2.f * y * gR[2][2]);
-        dq[3] = 2.f * (-2.f * z * gR[0][0] - w * gR[0][1] + x * gR[0][2] + w * gR[1][0] - 2.f * z * gR[1][1] +
-                       y * gR[1][2] + x * gR[2][0] + y * gR[2][1]);
-        const float dot = w * dq[0] + x * dq[1] + y * dq[2] + z * dq[3];
-        const float iqn = 1.f / o.qn;
-        gq[0] += (dq[0] - w * dot) * iqn;
-        gq[1] += (dq[1] - x * dot) * iqn;
-        gq[2] += (dq[2] - y * dot) * iqn;
-        gq[3] += (dq[3] - z * dot) * iqn;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float s2 = 2.f * frame.s[k] * frame.s[k];
+        gls[k] *= s2;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) gR[r][k] *= s2;
+    }
+    // R(q) of the normalised quaternion, then d(q / |q|)
+    const float w = frame.qw, x = frame.qx, y = frame.qy, z = frame.qz;
+    float dq[4];
+    dq[0] = 2.f * (-z * gR[0][1] + y * gR[0][2] + z * gR[1][0] - x * gR[1][2] - y * gR[2][0] + x * gR[2][1]);
+    dq[1] = 2.f * (y * gR[0][1] + z * gR[0][2] + y * gR[1][0] - 2.f * x * gR[1][1] - w * gR[1][2] + z * gR[2][0] +
+                   w * gR[2][1] - 2.f * x * gR[2][2]);
+    dq[2] = 2.f * (-2.f * y * gR[0][0] + x * gR[0][1] + w * gR[0][2] + x * gR[1][0] + z * gR[1][2] -
+                   w * gR[2][0] + z * gR[2][1] - 2.f * y * gR[2][2]);
+    dq[3] = 2.f * (-2.f * z * gR[0][0] - w * gR[0][1] + x * gR[0][2] + w * gR[1][0] - 2.f * z * gR[1][1] +
+                   y * gR[1][2] + x * gR[2][0] + y * gR[2][1]);
+    const float dot = w * dq[0] + x * dq[1] + y * dq[2] + z * dq[3];
+    const float iqn = 1.f / frame.qn;
+    const float gq[4] = {(dq[0] - w * dot) * iqn, (dq[1] - x * dot) * iqn, (dq[2] - y * dot) * iqn,
+                         (dq[3] - z * dot) * iqn};
+    if (!seen) {  // zero, whatever its scales and quaternion are
+#pragma unroll
+        for (int k = 0; k < 3; ++k) dL_dmeans3D[3 * g + k] = dL_dlog_scales[3 * g + k] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dL_dquats[4 * g + k] = 0.f;
+        return;
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -314,6 +355,7 @@ static CamDev cam_dev(const bgs_camera &c, int tile_w, int tile_h) {
     cam.lim_y = 1.3f * (float)((double)c.height / (2.0 * (double)c.fy));
     cam.W = c.width; cam.H = c.height;
     cam.tile_w = tile_w; cam.tile_h = tile_h;
+    cam.inv_tw = tile_recip(tile_w); cam.inv_th = tile_recip(tile_h);
     cam.tiles_x = (c.width + tile_w - 1) / tile_w;
     cam.tiles_y = (c.height + tile_h - 1) / tile_h;
     return cam;
@@ -328,7 +370,7 @@ cudaError_t launch_preprocess(long long N, int V, const float *means3D, const fl
     ct.V = V;
     for (int v = 0; v < V; ++v) ct.cam[v] = cam_dev(cams[v], tile_w, tile_h);
     if (N == 0) return cudaSuccess;
-    const int threads = 256;
+    const int threads = 128;
     const long long blocks = (N + threads - 1) / threads;
     k_preprocess<<<(unsigned)blocks, threads, 0, s>>>(N, means3D, log_scales, quats, opacities, ct,
                                                        reinterpret_cast<float2 *>(means2D),
@@ -346,7 +388,7 @@ cudaError_t launch_preprocess_backward(long long N, int V, const float *means3D,
     ct.V = V;
     for (int v = 0; v < V; ++v) ct.cam[v] = cam_dev(cams[v], 16, 16);
     if (N == 0) return cudaSuccess;
-    k_preprocess_backward<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(
+    k_preprocess_backward<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(
         N, means3D, log_scales, quats, ct, radii, reinterpret_cast<const float2 *>(dL_dmeans2D), dL_dconic,
         dL_ddepths, dL_dmeans3D, dL_dlog_scales, dL_dquats);
     return cudaGetLastError();
@@ -386,7 +428,7 @@ __global__ void __launch_bounds__(256) k_touched(long long N, const float2 *__re
     if (r > 0) {
         const float2 m = means2D[i];
         int x0, x1, y0, y1;
-        tile_rect(m.x, m.y, r, tw, th, tx, ty, x0, x1, y0, y1);
+        tile_rect(m.x, m.y, r, tw, th, tile_recip(tw), tile_recip(th), tx, ty, x0, x1, y0, y1);
         if (x1 > x0 && y1 > y0) c = (uint32_t)((x1 - x0) * (y1 - y0));
     }
     touched[i] = c;
@@ -436,7 +478,7 @@ __global__ void __launch_bounds__(256) k_duplicate(long long N, const uint32_t *
         if (r > 0) {
             const float2 m = means2D[i];
             int x1, y1;
-            tile_rect(m.x, m.y, r, tw, th, tx, ty, x0, x1, y0, y1);
+            tile_rect(m.x, m.y, r, tw, th, tile_recip(tw), tile_recip(th), tx, ty, x0, x1, y0, y1);
             if (x1 > x0 && y1 > y0) {
                 w = x1 - x0;
                 cnt = w * (y1 - y0);
