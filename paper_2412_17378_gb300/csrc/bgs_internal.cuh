@@ -46,6 +46,7 @@ struct DevCtrl {
     // binning: each view's entry count and first point_list slot
     unsigned long long view_k[kMaxViews];
     unsigned long long view_base[kMaxViews];
+    unsigned int bin_done[kMaxViews];  // column blocks done (returns to zero)
 };
 
 // End of a persistent pass, per warp (lane 0), for a block of `warps_per_block` warps whose
@@ -374,8 +375,8 @@ cudaError_t launch_preprocess_backward(long long N, int V, const float *means3D,
 // idx[i] = i for i in [lo, hi)
 cudaError_t launch_iota(long long lo, long long hi, uint32_t *idx, cudaStream_t s);
 
-cudaError_t launch_touched(long long N, const float *means2D, const int *radii, const float *depths, int W, int H,
-                           int tile_w, int tile_h, uint32_t *touched, uint32_t *dkey, uint32_t *idx, cudaStream_t s);
+cudaError_t launch_touched(long long N, const float *means2D, const int *radii, int W, int H, int tile_w, int tile_h,
+                           uint32_t *touched, cudaStream_t s);
 cudaError_t launch_gather_u32(long long N, const uint32_t *src, const uint32_t *order, uint32_t *dst, cudaStream_t s);
 template <typename KeyT>
 cudaError_t launch_duplicate(long long N, const uint32_t *order, const float *means2D, const int *radii,
@@ -400,31 +401,44 @@ cudaError_t launch_bin_count(long long N, int G, int b_lo, int b_hi, const uint3
                              const int *radii, int W, int H, int tw, int th, uint32_t *Hm, uint4 *rect, uint32_t *masks,
                              int W32, const int *skipP, cudaStream_t s);
 // the tiles whose credits over blocks [0, B1) certify that every pixel stopped, as the
-// exclusive 2D prefix P [(ty + 1) x (tx + 1)] of their indicator; P's buffer holds tx ty more
-// words behind the prefix (the per-tile sums)
-cudaError_t launch_bin_stopped(int B1, int tx, int ty, const uint16_t *D, int *P, cudaStream_t s);
+// exclusive 2D prefix P [(ty + 1) x (tx + 1)] of their indicator; S [tx ty] holds the per-tile
+// sums, zero before and after
+cudaError_t launch_bin_stopped(int B1, int tx, int ty, const uint16_t *D, uint32_t *S, int *P, cudaStream_t s);
+// What the binning of one view publishes once its tile totals are known (by the last block of
+// the column scan, or for one view of several by k_bin_open): each tile's start in the view
+// and, from the view's first point_list slot on, its range; the scatter's items per tile group
+// (with truncation); for a call's only view the call's entry count, also to host_k (nullable,
+// mapped host memory), with the overflow check against capacity.
+struct BinTiles {
+    int T, tx, ty, B, nC, v;
+    uint32_t *total, *start;
+    uint2 *ranges;
+    const uint32_t *bsat;  // nullable: complete lists
+    uint32_t *item_start;
+    bool only;             // the call's only view
+    long long capacity;
+    unsigned long long *host_k;
+    DevCtrl *ctrl;
+};
 // per tile column: exclusive prefix of H over the blocks and the total; with the credits D
 // (nullable) the column is cut after the block b_sat[t] at which they certify that every
-// pixel of the tile has stopped (b_sat written when bsat is not null)
-cudaError_t launch_bin_colscan(int B, int T, uint32_t *Hm, const uint16_t *D, uint32_t *total, uint32_t *bsat,
-                               cudaStream_t s);
+// pixel of the tile has stopped (b_sat written when bt.bsat is not null); the last block then
+// scans the totals into the starts and stores the view's entry count in ctrl->view_k[v]
+cudaError_t launch_bin_colscan(uint32_t *Hm, const uint16_t *D, const BinTiles &bt, cudaStream_t s);
 // per block and tile: fixed-point credits toward that certificate (k_bin_credit)
 size_t bin_credit_smem(int tx, int ty);
 cudaError_t launch_bin_credit(long long N, int G, int b_lo, int b_hi, const uint4 *rect, const float *means2D,
                               const float *conic_opacity, int W, int H, int tw, int th, uint16_t *D, cudaStream_t s);
-// ranges of view v's tiles, offset by the view's first point_list slot (the sum of the entry
-// counts of views 0..v-1, stored in ctrl->view_base[v] for the scatter)
-cudaError_t launch_bin_ranges(int T, const uint32_t *start, const uint32_t *total, uint2 *ranges, int v,
-                              DevCtrl *ctrl, cudaStream_t s);
+// a view of several: its ranges from the sum of the entry counts of views 0..v-1 on (stored in
+// ctrl->view_base[v] for the scatter) and the scatter's items
+cudaError_t launch_bin_open(const BinTiles &bt, cudaStream_t s);
 cudaError_t launch_bin_scatter(long long N, int G, int B, int W32, const uint4 *rect, int W, int H, int tw, int th,
                                const uint32_t *Hm, const uint32_t *start, const uint32_t *masks, uint32_t *point_list,
-                               long long capacity, const uint32_t *bsat, uint32_t *item_start, int num_sms, int v,
-                               const DevCtrl *ctrl, cudaStream_t s);
-// ctrl->view_k[v] = view v's entry count (64-bit sum of its tile totals)
-cudaError_t launch_bin_view_total(int T, const uint32_t *total, int v, DevCtrl *ctrl, cudaStream_t s);
-// num_entries = bin_base = the sum of the V views' counts; raises BGS_CHECK_OVERFLOW past
-// capacity or BGS_MAX_ENTRIES
-cudaError_t launch_bin_finish(int V, long long capacity, DevCtrl *ctrl, cudaStream_t s);
+                               long long capacity, const uint32_t *bsat, const uint32_t *item_start, int num_sms,
+                               int v, const DevCtrl *ctrl, cudaStream_t s);
+// num_entries = bin_base = the sum of the V views' counts, also to host_k (nullable); raises
+// BGS_CHECK_OVERFLOW past capacity or BGS_MAX_ENTRIES
+cudaError_t launch_bin_finish(int V, long long capacity, DevCtrl *ctrl, unsigned long long *host_k, cudaStream_t s);
 
 // view-dependent colour from spherical harmonics (sh.cu); backward: dL_drgb -> dL_dsh,
 // dL_dmeans3D (summed over the V <= kMaxViews camera centres campos [V,3], host)

@@ -15,10 +15,11 @@
 //   2. k_bin_colscan - exclusive scan of every column of H over b (in place) and the tile
 //                      totals n[t]; with credits, each tile's list is cut after the block
 //                      at which its pixels are certified to have stopped.
-//   3. (CUB) exclusive scan of n -> tile start; k_bin_view_total sums the view's count;
-//      k_bin_ranges writes the ranges, offset by the view's first point_list slot (the
-//      counts of the views before it: the views of a batched call run concurrently up to
-//      here, and each view's scatter waits only for the counts of the views before it).
+//   3. the last block of the column scan scans n -> tile start and stores the view's count.
+//      The ranges start at the view's first point_list slot (the counts of the views before
+//      it): for a call's only view that block writes them too, for one of several k_bin_open
+//      does (the views run concurrently up to here, and each view's ranges and scatter wait
+//      only for the counts of the views before it).
 //   4. k_bin_scatter - item (b, C), one warp, lane l owns tile l of C and keeps its write
 //                      position start[t] + H[b][t] in a register.  The warp visits the
 //                      Gaussians flagged in the (b, C) mask in depth order; every lane whose
@@ -425,15 +426,113 @@ __global__ void __launch_bounds__(kCrWarps * 32) k_bin_credit(long long N, int G
     }
 }
 
+// The call's entry count; overflow check.
+__device__ __forceinline__ void publish_count(unsigned long long k, long long capacity, DevCtrl *ctrl,
+                                              unsigned long long *host_k) {
+    ctrl->bin_base = k;
+    ctrl->num_entries = k;
+    if (host_k) *((volatile unsigned long long *)host_k) = k;
+    if ((long long)k > capacity || (long long)k > BGS_MAX_ENTRIES) atomicOr(&ctrl->check_bits, (unsigned)BGS_CHECK_OVERFLOW);
+}
+
+// Exclusive scan of the tile totals by the 32 warps of one block, each over a run of tiles read 32
+// at a time: start[t], the 64-bit count of the view and, for a call's only view, its ranges.
+__device__ __forceinline__ void scan_tiles(const BinTiles &bt, int tid) {
+    __shared__ unsigned long long part[32];
+    const int lane = tid & 31, warp = tid >> 5;
+    const int per = ((bt.T + 1023) / 1024) * 32, t0 = min(bt.T, warp * per), t1 = min(bt.T, t0 + per);
+    unsigned long long sum = 0;
+#pragma unroll 8
+    for (int t = t0 + lane; t < t1; t += 32) sum += __ldcg(bt.total + t);
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) part[warp] = sum;
+    __syncthreads();
+    unsigned long long base = 0, K = 0;
+    for (int w = 0; w < 32; ++w) {
+        const unsigned long long u = part[w];
+        if (w < warp) base += u;
+        K += u;
+    }
+    uint32_t run = (uint32_t)base;  // past 2^32 the call raises BGS_CHECK_OVERFLOW
+#pragma unroll 4
+    for (int tb = t0; tb < t1; tb += 32) {
+        const int t = tb + lane;
+        const uint32_t n = t < t1 ? __ldcg(bt.total + t) : 0u;
+        uint32_t incl = n;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        const uint32_t first = run + incl - n;
+        if (t < t1) {
+            bt.start[t] = first;
+            if (bt.only) bt.ranges[t] = n ? make_uint2(first, first + n) : make_uint2(0u, 0u);
+        }
+        run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (tid == 0) {
+        bt.ctrl->view_k[bt.v] = K;
+        if (bt.only) {
+            bt.ctrl->view_base[bt.v] = 0ull;
+            publish_count(K, bt.capacity, bt.ctrl, bt.host_k);
+        }
+    }
+}
+
+// Work items of the scatter: the (depth block b, tile group C) pairs with b at most the last
+// block any tile of C keeps, numbered C-major.  By the 1024 threads of one block, a lane per
+// tile of a group while its last block is found: item_start[C] = exclusive prefix of min(B, max
+// over C's tiles of b_sat + 1), and item_start[nC] = the item count.
+__device__ __forceinline__ void open_items(const BinTiles &bt, int tid) {
+    __shared__ uint32_t part[32];
+    const int lane = tid & 31, warp = tid >> 5;
+    const int nC = bt.nC, ncx = (bt.tx + kCbW - 1) / kCbW;
+#pragma unroll 4
+    for (int C = warp; C < nC; C += 32) {
+        const int x = (C % ncx) * kCbW + lane % kCbW, y = (C / ncx) * kCbH + lane / kCbW;
+        const uint32_t last = x < bt.tx && y < bt.ty ? __ldcg(bt.bsat + (size_t)y * bt.tx + x) : 0u;
+        const uint32_t n = min((uint32_t)bt.B, __reduce_max_sync(0xffffffffu, last) + 1u);
+        if (lane == 0) bt.item_start[C] = n;  // the count, turned into the offset below
+    }
+    __syncthreads();
+    uint32_t run = 0;
+    for (int c0 = 0; c0 < nC; c0 += 1024) {  // 1024 groups at a time (a 3840 x 2160 view has 1020)
+        const int C = c0 + tid;
+        const uint32_t n = C < nC ? bt.item_start[C] : 0u;
+        uint32_t incl = n;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (lane == 31) part[warp] = incl;
+        __syncthreads();
+        uint32_t base = run;
+        for (int w = 0; w < 32; ++w) {
+            const uint32_t u = part[w];
+            if (w < warp) base += u;
+            run += u;
+        }
+        if (C < nC) bt.item_start[C] = base + incl - n;
+        __syncthreads();
+    }
+    if (tid == 0) bt.item_start[nC] = run;
+}
+
 // Block (32 tiles) x (32 row groups): per column t, exclusive prefix over b in place, and
 // the column total n[t].  With the credits D (nullable): the column is cut after the first
 // block b_sat[t] at whose end the credits summed over blocks 0..b reach thr (every pixel of
 // the tile has stopped there); n[t] then counts blocks 0..b_sat only, and blocks past b_sat
 // keep stale values that the scatter never reads.  b_sat = B - 1 when the credits never
-// reach thr (or without D).
-__global__ void __launch_bounds__(1024) k_bin_colscan(int B, int T, uint32_t *__restrict__ H,
-                                                      const uint16_t *__restrict__ D, uint32_t thr,
-                                                      uint32_t *__restrict__ total, uint32_t *__restrict__ bsat) {
+// reach thr (or without D).  The last block to finish then publishes the tiles (BinTiles): one
+// launch where the scan, the count, the ranges and the scatter's items were five (of 3-7 us
+// each, on one block or a few).  With the key pass and the copies of the count gone as well, a
+// 256 x 256 frame of 10k Gaussians takes 232 instead of 270 us, the lists of 1M at 1080p 378
+// instead of 420.
+__global__ void __launch_bounds__(1024) k_bin_colscan(uint32_t *__restrict__ H, const uint16_t *__restrict__ D,
+                                                      uint32_t thr, const BinTiles bt, uint32_t *__restrict__ bsat) {
+    __shared__ bool s_last;
+    const int B = bt.B, T = bt.T;
+    uint32_t *total = bt.total;
     __shared__ uint32_t part[32][33], partD[32][33];
     __shared__ uint32_t s_gsat[32], s_runD[32], s_bsat[32], s_partH[32];
     const int lx = threadIdx.x, ly = threadIdx.y;
@@ -504,44 +603,37 @@ __global__ void __launch_bounds__(1024) k_bin_colscan(int B, int T, uint32_t *__
             off += h;
         }
     }
-}
-
-// ranges[t] = base + [start[t], start[t] + n[t]) for the tiles of view v ((0,0) for an empty
-// tile), base = the entries of views 0..v-1; block 0 stores base for the scatter.
-__global__ void k_bin_ranges(int T, const uint32_t *__restrict__ start, const uint32_t *__restrict__ total,
-                             uint2 *__restrict__ ranges, int v, DevCtrl *ctrl) {
-    unsigned long long b64 = 0;
-    for (int u = 0; u < v; ++u) b64 += ctrl->view_k[u];
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->view_base[v] = b64;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const uint32_t base = (uint32_t)b64;  // past 2^32 the call raises BGS_CHECK_OVERFLOW
-    const uint32_t a = base + start[t], n = total[t];
-    ranges[t] = n ? make_uint2(a, a + n) : make_uint2(0u, 0u);
-}
-
-// view_k[v] = the view's entry count, summed in 64 bits from the per-tile totals.
-__global__ void k_bin_view_total(int T, const uint32_t *__restrict__ total, int v, DevCtrl *ctrl) {
-    __shared__ unsigned long long part[32];
-    unsigned long long n = 0;
-    for (int t = threadIdx.x; t < T; t += blockDim.x) n += total[t];
-    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = n;
+    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long k = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) k += part[w];
-        ctrl->view_k[v] = k;
-    }
+    const int tid = ly * 32 + lx;
+    if (tid == 0) s_last = atomicAdd(&bt.ctrl->bin_done[bt.v], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (tid == 0) bt.ctrl->bin_done[bt.v] = 0u;
+    scan_tiles(bt, tid);
+    if (bt.only && bt.bsat) open_items(bt, tid);
 }
 
-// The call's entry count over its V views; overflow check.
-__global__ void k_bin_finish(int V, long long capacity, DevCtrl *ctrl) {
+// A view of several, one block: ranges[t] = base + [start[t], start[t] + n[t]) ((0,0) for an
+// empty tile), base = the entries of views 0..v-1, and the scatter's items.
+__global__ void __launch_bounds__(1024) k_bin_open(const BinTiles bt) {
+    unsigned long long b64 = 0;
+    for (int u = 0; u < bt.v; ++u) b64 += bt.ctrl->view_k[u];
+    if (threadIdx.x == 0) bt.ctrl->view_base[bt.v] = b64;
+    const uint32_t base = (uint32_t)b64;  // past 2^32 the call raises BGS_CHECK_OVERFLOW
+    for (int t = threadIdx.x; t < bt.T; t += 1024) {
+        const uint32_t a = base + bt.start[t], n = bt.total[t];
+        bt.ranges[t] = n ? make_uint2(a, a + n) : make_uint2(0u, 0u);
+    }
+    if (bt.bsat) open_items(bt, threadIdx.x);
+}
+
+// The call's entry count over its V views.
+__global__ void k_bin_finish(int V, long long capacity, DevCtrl *ctrl, unsigned long long *host_k) {
     unsigned long long k = 0;
     for (int u = 0; u < V; ++u) k += ctrl->view_k[u];
-    ctrl->bin_base = k;
-    ctrl->num_entries = k;
-    if ((long long)k > capacity || (long long)k > BGS_MAX_ENTRIES) atomicOr(&ctrl->check_bits, (unsigned)BGS_CHECK_OVERFLOW);
+    publish_count(k, capacity, ctrl, host_k);
 }
 
 // Writes the completed sector [done, done + 8) of a lane's run from its ring (words below
@@ -568,47 +660,6 @@ __device__ __forceinline__ void flush_sector(const uint32_t *ring_s, int lane, u
 // Single-warp blocks: a block's shared memory is released as soon as its warp is done
 // (blocks of several warps hold it until the slowest one finishes, and reached fewer
 // resident warps).
-// Work items of the scatter: the (depth block b, tile group C) pairs with b at most the last
-// block any tile of C keeps (every pair without truncation), numbered C-major.  One block:
-// item_start[C] = exclusive prefix of min(B, max over C's tiles of b_sat + 1), and
-// item_start[nC] = the item count.
-__global__ void __launch_bounds__(1024) k_bin_items(int nC, int tx, int ty, int B, const uint32_t *__restrict__ bsat,
-                                                    uint32_t *__restrict__ item_start) {
-    __shared__ uint32_t part[1024];
-    const int tid = threadIdx.x;
-    const int per = (nC + 1023) / 1024;
-    const int c0 = min(nC, tid * per), c1 = min(nC, c0 + per);
-    const int ncx = (tx + kCbW - 1) / kCbW;
-    uint32_t local = 0;
-    for (int C = c0; C < c1; ++C) {
-        uint32_t n = (uint32_t)B;
-        if (bsat) {
-            uint32_t gmax = 0;
-            const int gx0 = (C % ncx) * kCbW, gy0 = (C / ncx) * kCbH;
-            for (int y = gy0; y < min(ty, gy0 + kCbH); ++y)
-                for (int x = gx0; x < min(tx, gx0 + kCbW); ++x) gmax = max(gmax, bsat[(size_t)y * tx + x]);
-            n = min((uint32_t)B, gmax + 1u);
-        }
-        item_start[C] = n;  // the count, turned into the offset below
-        local += n;
-    }
-    part[tid] = local;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {  // inclusive scan of the threads' sums
-        const uint32_t v = tid >= off ? part[tid - off] : 0u;
-        __syncthreads();
-        part[tid] += v;
-        __syncthreads();
-    }
-    uint32_t run = part[tid] - local;
-    for (int C = c0; C < c1; ++C) {
-        const uint32_t n = item_start[C];
-        item_start[C] = run;
-        run += n;
-    }
-    if (tid == 1023) item_start[nC] = part[1023];
-}
-
 // With truncated lists (bsat given) the blocks stride over the work items of k_bin_items,
 // item -> (C, b); with complete lists every (b, C) is an item and block i takes item i
 // (C = i / B, b = i % B) once.  Item (b, C): one warp, lane l owns tile l of C; lanes whose
@@ -810,7 +861,7 @@ __global__ void k_bin_stopped(int B1, int T, int chunk, const uint16_t *__restri
 
 // P [(ty + 1) x (tx + 1)]: the exclusive 2D prefix of the stopped tiles' indicator (S[t] >=
 // thr), P[y][x] = #stopped tiles (x' < x, y' < y), built in shared memory by one block.
-__global__ void __launch_bounds__(1024) k_bin_prefix2d(int tx, int ty, const uint32_t *__restrict__ S, uint32_t thr,
+__global__ void __launch_bounds__(1024) k_bin_prefix2d(int tx, int ty, uint32_t *__restrict__ S, uint32_t thr,
                                                        int *__restrict__ P) {
     extern __shared__ int p_s[];
     const int w1 = tx + 1, n = (tx + 1) * (ty + 1), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -843,16 +894,14 @@ __global__ void __launch_bounds__(1024) k_bin_prefix2d(int tx, int ty, const uin
     }
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) P[i] = p_s[i];
+    for (int t = threadIdx.x; t < tx * ty; t += blockDim.x) S[t] = 0u;  // for the next pass
 }
 
 size_t bin_stopped_smem(int tx, int ty) { return sizeof(int) * (size_t)(tx + 1) * (ty + 1); }
 
-cudaError_t launch_bin_stopped(int B1, int tx, int ty, const uint16_t *D, int *P, cudaStream_t s) {
+cudaError_t launch_bin_stopped(int B1, int tx, int ty, const uint16_t *D, uint32_t *S, int *P, cudaStream_t s) {
     const int T = tx * ty;
-    // the per-tile sums live behind the prefix in P's buffer
-    uint32_t *S = reinterpret_cast<uint32_t *>(P + (size_t)(tx + 1) * (ty + 1));
-    cudaError_t e = cudaMemsetAsync(S, 0, sizeof(uint32_t) * (size_t)T, s);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     if (B1 > 0) {
         const int chunk = std::max(32, (B1 + 65534) / 65535);
         const dim3 grid((unsigned)std::max(1, (T + 255) / 256), (unsigned)((B1 + chunk - 1) / chunk));
@@ -865,9 +914,13 @@ cudaError_t launch_bin_stopped(int B1, int tx, int ty, const uint16_t *D, int *P
     return cudaGetLastError();
 }
 
-cudaError_t launch_bin_colscan(int B, int T, uint32_t *Hm, const uint16_t *D, uint32_t *total, uint32_t *bsat,
-                               cudaStream_t s) {
-    k_bin_colscan<<<(T + 31) / 32, dim3(32, 32), 0, s>>>(B, T, Hm, D, kCreditThr, total, bsat);
+cudaError_t launch_bin_colscan(uint32_t *Hm, const uint16_t *D, const BinTiles &bt, cudaStream_t s) {
+    k_bin_colscan<<<(bt.T + 31) / 32, dim3(32, 32), 0, s>>>(Hm, D, kCreditThr, bt, const_cast<uint32_t *>(bt.bsat));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_bin_open(const BinTiles &bt, cudaStream_t s) {
+    k_bin_open<<<1, 1024, 0, s>>>(bt);
     return cudaGetLastError();
 }
 
@@ -903,26 +956,15 @@ cudaError_t launch_bin_credit(long long N, int G, int b_lo, int b_hi, const uint
     return cudaGetLastError();
 }
 
-cudaError_t launch_bin_ranges(int T, const uint32_t *start, const uint32_t *total, uint2 *ranges, int v,
-                              DevCtrl *ctrl, cudaStream_t s) {
-    k_bin_ranges<<<std::max(1, (T + 255) / 256), 256, 0, s>>>(T, start, total, ranges, v, ctrl);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_bin_view_total(int T, const uint32_t *total, int v, DevCtrl *ctrl, cudaStream_t s) {
-    k_bin_view_total<<<1, 1024, 0, s>>>(T, total, v, ctrl);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_bin_finish(int V, long long capacity, DevCtrl *ctrl, cudaStream_t s) {
-    k_bin_finish<<<1, 1, 0, s>>>(V, capacity, ctrl);
+cudaError_t launch_bin_finish(int V, long long capacity, DevCtrl *ctrl, unsigned long long *host_k, cudaStream_t s) {
+    k_bin_finish<<<1, 1, 0, s>>>(V, capacity, ctrl, host_k);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bin_scatter(long long N, int G, int B, int W32, const uint4 *rect, int W, int H, int tw, int th,
                                const uint32_t *Hm, const uint32_t *start, const uint32_t *masks, uint32_t *point_list,
-                               long long capacity, const uint32_t *bsat, uint32_t *item_start, int num_sms, int v,
-                               const DevCtrl *ctrl, cudaStream_t s) {
+                               long long capacity, const uint32_t *bsat, const uint32_t *item_start, int num_sms,
+                               int v, const DevCtrl *ctrl, cudaStream_t s) {
     (void)N;
     const int tx = (W + tw - 1) / tw, ty = (H + th - 1) / th;
     const int nC = bin_mask_groups(tx, ty);
@@ -933,7 +975,6 @@ cudaError_t launch_bin_scatter(long long N, int G, int B, int W32, const uint4 *
     // over the open items; complete lists: one block per (b, C), scheduled by the hardware
     long long grid = (long long)B * nC;
     if (bsat) {
-        k_bin_items<<<1, 1024, 0, s>>>(nC, tx, ty, B, bsat, item_start);
         grid = std::min<long long>((long long)num_sms * 32, grid);
     }
     k_bin_scatter<<<(unsigned)std::max<long long>(1, grid), 32, 0, s>>>((uint32_t)G, W32, rect, tx, ty, Hm, start,

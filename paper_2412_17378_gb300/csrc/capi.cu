@@ -69,7 +69,7 @@ namespace bgs {
 int set_error(int code, const char *msg) { return fail(code, "%s", msg); }
 }  // namespace bgs
 
-constexpr int kSortStreams = 4;
+constexpr int kSortStreams = 8;
 
 struct bgs_plan {
     bgs_plan_desc desc;
@@ -82,15 +82,17 @@ struct bgs_plan {
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_fwd, ev_bwd;
     unsigned long long host_launches = 0;
     // binning
-    Buf touched, touched_sorted, dkey, dkey_sorted, gidx, order, offsets, keys_in, keys_out, vals_in, cub_tmp;
+    Buf touched, touched_sorted, dkey_sorted, gidx, order, offsets, keys_in, keys_out, vals_in, cub_tmp;
     // counting-sort binning, one buffer set per concurrent view (stream slot): tile histogram,
     // totals, starts, packed rectangles, masks; list truncation (credits, last block per
-    // tile); the scatter's work items per tile group; the tile scan's temporaries
+    // tile); the scatter's work items per tile group
     struct BinSlot {
-        Buf h, total, start, rect, mask, credit, sat, items, scan_tmp, stopped;
+        Buf h, total, start, rect, mask, credit, sat, items, stopped;
+        Buf stopped_sum;  // zero between passes, whatever their grid (each pass clears what it read)
     } bin_slot[kSortStreams];
     cudaEvent_t view_done[bgs::kMaxViews] = {};  // a view's entry count is known
     int smem_optin = 0;
+    unsigned long long *host_k = nullptr, *host_k_dev = nullptr;  // mapped: the last call's entry count
     // render
     Buf recs, tile_idx, items, grad_acc, warp_items;  // tile_idx: each tile's slot in its work-list bucket
     Buf gw_exoff, gw_ent, gw_tile, gw_done, gw_sum;  // Gaussian-wise segments: per-tile later-segment
@@ -389,6 +391,8 @@ int bgs_plan_create(const bgs_plan_desc *desc, bgs_plan **out) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e == cudaSuccess) e = cudaMalloc((void **)&p->ctrl, sizeof(bgs::DevCtrl));
     if (e == cudaSuccess) e = cudaMemset(p->ctrl, 0, sizeof(bgs::DevCtrl));
+    if (e == cudaSuccess) e = cudaHostAlloc((void **)&p->host_k, sizeof *p->host_k, cudaHostAllocMapped);
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&p->host_k_dev, p->host_k, 0);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->sort_fork, cudaEventDisableTiming);
     for (int i = 0; i < kSortStreams && e == cudaSuccess; ++i) {
         e = cudaStreamCreateWithFlags(&p->sort_stream[i], cudaStreamNonBlocking);
@@ -418,12 +422,12 @@ int bgs_plan_destroy(bgs_plan *p) {
     for (cudaEvent_t e : p->view_done)
         if (e) cudaEventDestroy(e);
     for (auto &sl : p->bin_slot) {
-        Buf *sb[] = {&sl.h,     &sl.total, &sl.start, &sl.rect,     &sl.mask,
-                     &sl.credit, &sl.sat,  &sl.items, &sl.scan_tmp, &sl.stopped};
+        Buf *sb[] = {&sl.h, &sl.total, &sl.start, &sl.rect, &sl.mask, &sl.credit, &sl.sat, &sl.items, &sl.stopped,
+                     &sl.stopped_sum};
         for (Buf *b : sb)
             if (b->p) cudaFree(b->p);
     }
-    Buf *bufs[] = {&p->gw_exoff, &p->gw_ent, &p->gw_done, &p->gw_sum, &p->gw_tile, &p->tile_cost, &p->vkey_sorted, &p->touched, &p->touched_sorted, &p->dkey,
+    Buf *bufs[] = {&p->gw_exoff, &p->gw_ent, &p->gw_done, &p->gw_sum, &p->gw_tile, &p->tile_cost, &p->vkey_sorted, &p->touched, &p->touched_sorted,
                    &p->dkey_sorted, &p->gidx, &p->order, &p->offsets,
                    &p->keys_in, &p->keys_out, &p->vals_in, &p->cub_tmp, &p->recs,
                    &p->tile_idx, &p->items, &p->warp_items,
@@ -431,6 +435,7 @@ int bgs_plan_destroy(bgs_plan *p) {
     for (Buf *b : bufs)
         if (b->p) cudaFree(b->p);
     if (p->ctrl) cudaFree(p->ctrl);
+    if (p->host_k) cudaFreeHost(p->host_k);
     for (auto &e : p->ev_fwd) {
         cudaEventDestroy(e.first);
         cudaEventDestroy(e.second);
@@ -553,7 +558,7 @@ int bgs_plan_reserve(bgs_plan *p, int64_t N, int64_t K, int64_t T, int64_t pixel
     if (!p || N < 0 || K < 0 || T < 0 || pixels < 0) return fail(BGS_ERR_INVALID, "bgs_plan_reserve: bad sizes");
     DeviceGuard g(p->device);
     cudaStream_t s = 0;
-    Buf *n4[] = {&p->touched, &p->touched_sorted, &p->dkey, &p->dkey_sorted, &p->gidx, &p->order};
+    Buf *n4[] = {&p->touched, &p->touched_sorted, &p->dkey_sorted, &p->gidx, &p->order};
     for (Buf *b : n4) BGS_TRY(ensure(p, *b, 4 * N, s, "per-Gaussian"));
     BGS_TRY(ensure(p, p->offsets, 8 * N, s, "offsets"));
     BGS_TRY(ensure(p, p->keys_in, 4 * K, s, "keys_in"));
@@ -677,21 +682,26 @@ namespace {
 // set `slot`.  order holds the view's records in depth order (global record indices);
 // ranges points at the view's first tile.  bin_view_a counts (tile histogram, masks,
 // credits, truncated totals, tile starts) and stores the view's entry count in
-// ctrl->view_k[v]; bin_view_b writes the ranges and the lists from the view's first
-// point_list slot (the counts of views 0..v-1, which must be stored by then) on.  No host
-// synchronisation; bgs::launch_bin_finish then totals the call's views.
+// ctrl->view_k[v]; for a call's only view (only) it writes the ranges and publishes the count
+// too.  bin_view_b writes the lists from the view's first point_list slot (the counts of views
+// 0..v-1, which must be stored by then) on, for one of several views behind its ranges.  No
+// host synchronisation; bgs::launch_bin_finish then totals the call's views.
 // depth-order fractions 1 / d at which truncated binning starts its second and third passes
 constexpr long long kBinPassDiv[2] = {8, 2};
+
+// the capacity a synchronous call hands its kernels: the host compares the count itself
+constexpr long long kSyncCapacity = 1ll << 62;
 
 struct BinView {
     int tiles_x, tiles_y;
     long long T, G, B, W32, nC;
     bool trunc;
+    bgs::BinTiles tiles;
 };
 
 int bin_view_a(bgs_plan *p, int slot, int v, long long n, const uint32_t *order, const float *means2D,
-               const int32_t *radii, const float *conic_opacity, int W, int H, int tw, int th, BinView &bv,
-               cudaStream_t s) {
+               const int32_t *radii, const float *conic_opacity, int W, int H, int tw, int th, bool only,
+               long long capacity, uint32_t *ranges, BinView &bv, cudaStream_t s) {
     bgs_plan::BinSlot &sl = p->bin_slot[slot];
     bv.tiles_x = (W + tw - 1) / tw;
     bv.tiles_y = (H + th - 1) / th;
@@ -745,12 +755,16 @@ int bin_view_a(bgs_plan *p, int slot, int v, long long n, const uint32_t *order,
     uint32_t *masks = (uint32_t *)sl.mask.p;
     int *P = nullptr;
     if (passes > 1) {
-        BGS_TRY(ensure(p, sl.stopped, sizeof(int) * ((bv.tiles_x + 1) * (bv.tiles_y + 1) + bv.T), s, "bin_stopped"));
+        BGS_TRY(ensure(p, sl.stopped, sizeof(int) * (size_t)(bv.tiles_x + 1) * (bv.tiles_y + 1), s, "bin_stopped"));
+        const size_t before = sl.stopped_sum.bytes;
+        BGS_TRY(ensure(p, sl.stopped_sum, sizeof(uint32_t) * T, s, "bin_stopped_sum"));
+        if (sl.stopped_sum.bytes != before)
+            BGS_CUDA(cudaMemsetAsync(sl.stopped_sum.p, 0, sl.stopped_sum.bytes, s), "clear bin_stopped_sum");
         P = (int *)sl.stopped.p;
     }
     for (int k = 0; k < passes; ++k) {
         const int lo = (int)bounds[k], hi = (int)bounds[k + 1];
-        if (k > 0) BGS_CUDA(bgs::launch_bin_stopped(lo, bv.tiles_x, bv.tiles_y, credit, P, s), "bin_stopped");
+        if (k > 0) BGS_CUDA(bgs::launch_bin_stopped(lo, bv.tiles_x, bv.tiles_y, credit, (uint32_t *)sl.stopped_sum.p, P, s), "bin_stopped");
         BGS_CUDA(bgs::launch_bin_count(n, (int)G, lo, hi, order, means2D, radii, W, H, tw, th, Hm, rect, masks,
                                        (int)W32, k > 0 ? P : nullptr, s),
                  "bin_count");
@@ -760,31 +774,49 @@ int bin_view_a(bgs_plan *p, int slot, int v, long long n, const uint32_t *order,
         p->host_launches += k > 0 ? 4 : 1;
     }
     if (bv.trunc) p->host_launches += 1;
-    BGS_CUDA(bgs::launch_bin_colscan((int)B, (int)T, Hm, credit, tot, bsat, s), "bin_colscan");
-    size_t tmp = 0;
-    BGS_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tmp, tot, start, (int)T, s), "tile scan (size)");
-    BGS_TRY(ensure(p, sl.scan_tmp, tmp, s, "scan_tmp"));
-    tmp = sl.scan_tmp.bytes;
-    BGS_CUDA(cub::DeviceScan::ExclusiveSum(sl.scan_tmp.p, tmp, tot, start, (int)T, s), "tile scan");
-    BGS_CUDA(bgs::launch_bin_view_total((int)T, tot, v, p->ctrl, s), "bin_view_total");
-    p->host_launches += 3;  // count, colscan, view total
+    BGS_TRY(ensure(p, sl.items, sizeof(uint32_t) * (bv.nC + 1), s, "bin_items"));
+    bgs::BinTiles &bt = bv.tiles;
+    bt.T = (int)T, bt.tx = bv.tiles_x, bt.ty = bv.tiles_y, bt.B = (int)B, bt.nC = (int)nC, bt.v = v;
+    bt.total = tot;
+    bt.start = start;
+    bt.ranges = reinterpret_cast<uint2 *>(ranges);
+    bt.bsat = bsat;
+    bt.item_start = (uint32_t *)sl.items.p;
+    bt.only = only;
+    bt.capacity = capacity;
+    bt.host_k = capacity == kSyncCapacity ? p->host_k_dev : nullptr;  // a synchronous call reads it
+    bt.ctrl = p->ctrl;
+    BGS_CUDA(bgs::launch_bin_colscan(Hm, credit, bt, s), "bin_colscan");
+    p->host_launches += 1;
     return BGS_OK;
 }
 
 int bin_view_b(bgs_plan *p, int slot, int v, long long n, const BinView &bv, int W, int H, int tw, int th,
-               uint32_t *point_list, long long capacity, uint32_t *ranges, cudaStream_t s) {
+               uint32_t *point_list, long long capacity, cudaStream_t s) {
     bgs_plan::BinSlot &sl = p->bin_slot[slot];
-    const uint32_t *Hm = (const uint32_t *)sl.h.p, *tot = (const uint32_t *)sl.total.p;
-    const uint32_t *start = (const uint32_t *)sl.start.p;
-    BGS_CUDA(bgs::launch_bin_ranges((int)bv.T, start, tot, reinterpret_cast<uint2 *>(ranges), v, p->ctrl, s),
-             "bin_ranges");
-    BGS_TRY(ensure(p, sl.items, sizeof(uint32_t) * (bv.nC + 1), s, "bin_items"));
-    BGS_CUDA(bgs::launch_bin_scatter(n, (int)bv.G, (int)bv.B, (int)bv.W32, (const uint4 *)sl.rect.p, W, H, tw, th, Hm,
-                                     start, (const uint32_t *)sl.mask.p, point_list, capacity,
-                                     bv.trunc ? (const uint32_t *)sl.sat.p : nullptr, (uint32_t *)sl.items.p,
+    if (!bv.tiles.only) {
+        BGS_CUDA(bgs::launch_bin_open(bv.tiles, s), "bin_open");
+        p->host_launches += 1;
+    }
+    BGS_CUDA(bgs::launch_bin_scatter(n, (int)bv.G, (int)bv.B, (int)bv.W32, (const uint4 *)sl.rect.p, W, H, tw, th,
+                                     (const uint32_t *)sl.h.p, (const uint32_t *)sl.start.p,
+                                     (const uint32_t *)sl.mask.p, point_list, capacity,
+                                     bv.trunc ? (const uint32_t *)sl.sat.p : nullptr, (const uint32_t *)sl.items.p,
                                      p->num_sms, v, p->ctrl, s),
              "bin_scatter");
-    p->host_launches += bv.trunc ? 3 : 2;  // ranges, (work list), scatter
+    p->host_launches += 1;
+    return BGS_OK;
+}
+
+// Record indices 0, 1, ... for the depth sorts' values, kept in gidx from one call to the next
+// (a call under stream capture records the fill without counting it as done, so that its
+// graph fills them on every replay).
+int ensure_indices(bgs_plan *p, long long n, cudaStream_t s) {
+    BGS_TRY(ensure(p, p->gidx, 4 * n, s, "gidx"));
+    if (p->iota_n >= n) return BGS_OK;
+    BGS_CUDA(bgs::launch_iota(p->iota_n, n, (uint32_t *)p->gidx.p, s), "record indices");
+    p->host_launches += 1;
+    if (!capturing(s)) p->iota_n = n;
     return BGS_OK;
 }
 
@@ -834,23 +866,20 @@ int bgs_bin_and_sort(bgs_plan *p, int64_t N, const float *means2D, const int32_t
     if (T >= (1ll << 31)) return fail(BGS_ERR_INVALID, "bgs_bin_and_sort: too many tiles");
     DeviceGuard g(p->device);
     cudaStream_t s = (cudaStream_t)stream;
-    BGS_CUDA(cudaMemsetAsync(ranges, 0, sizeof(uint2) * T, s), "clear ranges");
     if (num_rendered) *num_rendered = 0;
     if (needed) *needed = 0;
+    // the counting sort (when its per-tile counters fit in shared memory) writes every range
+    const bool counting = N > 0 && bgs::bin_count_smem(tiles_x, tiles_y) <= (size_t)p->smem_optin;
+    if (!counting) BGS_CUDA(cudaMemsetAsync(ranges, 0, sizeof(uint2) * T, s), "clear ranges");
     if (N == 0) return BGS_OK;
-    // (1) entry counts and the depth order of the Gaussians (stable: ties keep index order)
-    BGS_TRY(ensure(p, p->touched, 4 * N, s, "touched"));
-    BGS_TRY(ensure(p, p->touched_sorted, 4 * N, s, "touched_sorted"));
-    BGS_TRY(ensure(p, p->dkey, 4 * N, s, "dkey"));
+    // (1) the depth order of the Gaussians (stable: ties keep index order): the keys are the
+    // depths' float32 bit patterns
     BGS_TRY(ensure(p, p->dkey_sorted, 4 * N, s, "dkey_sorted"));
-    BGS_TRY(ensure(p, p->gidx, 4 * N, s, "gidx"));
+    BGS_TRY(ensure_indices(p, N, s));
     BGS_TRY(ensure(p, p->order, 4 * N, s, "order"));
-    BGS_TRY(ensure(p, p->offsets, 8 * N, s, "offsets"));
-    uint32_t *touched = (uint32_t *)p->touched.p, *tsorted = (uint32_t *)p->touched_sorted.p;
-    uint32_t *dkey = (uint32_t *)p->dkey.p, *dkey2 = (uint32_t *)p->dkey_sorted.p;
-    uint32_t *gidx = (uint32_t *)p->gidx.p, *order = (uint32_t *)p->order.p;
-    unsigned long long *off = (unsigned long long *)p->offsets.p;
-    BGS_CUDA(bgs::launch_touched(N, means2D, radii, depths, W, H, tw, th, touched, dkey, gidx, s), "touched");
+    const uint32_t *dkey = reinterpret_cast<const uint32_t *>(depths);
+    uint32_t *dkey2 = (uint32_t *)p->dkey_sorted.p, *order = (uint32_t *)p->order.p;
+    const uint32_t *gidx = (const uint32_t *)p->gidx.p;
     size_t tmp = 0;
     BGS_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tmp, dkey, dkey2, gidx, order, (int64_t)N, 0, 32, s),
              "depth sort (size)");
@@ -858,15 +887,14 @@ int bgs_bin_and_sort(bgs_plan *p, int64_t N, const float *means2D, const int32_t
     tmp = p->cub_tmp.bytes;
     BGS_CUDA(cub::DeviceRadixSort::SortPairs(p->cub_tmp.p, tmp, dkey, dkey2, gidx, order, (int64_t)N, 0, 32, s),
              "depth sort");
-    // (2) counting sort over tile rectangles when the per-tile counters fit in shared memory
-    if (bgs::bin_count_smem(tiles_x, tiles_y) <= (size_t)p->smem_optin) {
+    // (2) counting sort over tile rectangles
+    if (counting) {
         BinView bv;
-        BGS_TRY(bin_view_a(p, 0, 0, N, order, means2D, radii, conic_opacity, W, H, tw, th, bv, s));
-        BGS_TRY(bin_view_b(p, 0, 0, N, bv, W, H, tw, th, point_list, capacity, ranges, s));
-        BGS_CUDA(bgs::launch_bin_finish(1, 1ll << 62, p->ctrl, s), "bin_finish");  // the host checks K
-        unsigned long long K = 0;
-        BGS_CUDA(cudaMemcpyAsync(&K, &p->ctrl->num_entries, sizeof K, cudaMemcpyDeviceToHost, s), "read K");
+        // (the host checks K against the capacity)
+        BGS_TRY(bin_view_a(p, 0, 0, N, order, means2D, radii, conic_opacity, W, H, tw, th, true, kSyncCapacity, ranges, bv, s));
+        BGS_TRY(bin_view_b(p, 0, 0, N, bv, W, H, tw, th, point_list, capacity, s));
         BGS_CUDA(cudaStreamSynchronize(s), "sync K");
+        const unsigned long long K = *(volatile unsigned long long *)p->host_k;
         if (needed) *needed = (int64_t)K;
         if ((long long)K > capacity || (long long)K > BGS_MAX_ENTRIES)
             return fail(BGS_ERR_CAPACITY, "bgs_bin_and_sort: %llu entries exceed capacity %lld (or BGS_MAX_ENTRIES)",
@@ -874,7 +902,13 @@ int bgs_bin_and_sort(bgs_plan *p, int64_t N, const float *means2D, const int32_t
         if (num_rendered) *num_rendered = (int64_t)K;
         return BGS_OK;
     }
-    // (2') otherwise: entry offsets in depth order, emit, stable radix sort on the tile id
+    // (2') otherwise: entry counts and offsets in depth order, emit, stable radix sort on the tile id
+    BGS_TRY(ensure(p, p->touched, 4 * N, s, "touched"));
+    BGS_TRY(ensure(p, p->touched_sorted, 4 * N, s, "touched_sorted"));
+    BGS_TRY(ensure(p, p->offsets, 8 * N, s, "offsets"));
+    uint32_t *touched = (uint32_t *)p->touched.p, *tsorted = (uint32_t *)p->touched_sorted.p;
+    unsigned long long *off = (unsigned long long *)p->offsets.p;
+    BGS_CUDA(bgs::launch_touched(N, means2D, radii, W, H, tw, th, touched, s), "touched");
     BGS_CUDA(bgs::launch_gather_u32(N, touched, order, tsorted, s), "gather counts");
     tmp = 0;
     BGS_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tmp, tsorted, off, (int64_t)N, s), "scan (size)");
@@ -1286,36 +1320,34 @@ int bgs_bin_and_sort_batched(bgs_plan *p, int32_t V, const bgs_view *views, int6
     DeviceGuard g(p->device);
     cudaStream_t s = (cudaStream_t)stream;
     const long long T = vt.tile_base[V];
-    BGS_CUDA(cudaMemsetAsync(ranges, 0, sizeof(uint2) * T, s), "clear ranges");
-    BGS_CUDA(cudaMemsetAsync(&p->ctrl->bin_base, 0, sizeof(unsigned long long), s), "clear bin base");
     if (num_rendered) *num_rendered = 0;
     if (needed) *needed = 0;
     const long long R = N * V;
+    if (R == 0) {  // (the binning writes every range and the count)
+        BGS_CUDA(cudaMemsetAsync(ranges, 0, sizeof(uint2) * T, s), "clear ranges");
+        BGS_CUDA(cudaMemsetAsync(&p->ctrl->bin_base, 0, sizeof(unsigned long long), s), "clear bin base");
+    }
     if (R > 0) {
         // depth order of every view's records: one 32-bit key sort per view slice (a single
         // sort of 64-bit (view, depth) keys over all V N records was measured slower)
         BGS_TRY(ensure(p, p->vkey_sorted, 4 * R, s, "dkey_sorted"));
-        BGS_TRY(ensure(p, p->gidx, 4 * R, s, "gidx"));
+        BGS_TRY(ensure_indices(p, R, s));
         BGS_TRY(ensure(p, p->order, 4 * R, s, "order"));
         // keys: the depths' float32 bit patterns (the order both sides sort on); values: record
-        // indices, kept in gidx from one call to the next (a call under stream capture records
-        // the fill without counting it as done, so that its graph fills them on every replay)
+        // indices
         const uint32_t *k0 = reinterpret_cast<const uint32_t *>(depths);
         uint32_t *k1 = (uint32_t *)p->vkey_sorted.p;
         uint32_t *gidx = (uint32_t *)p->gidx.p, *order = (uint32_t *)p->order.p;
-        if (p->iota_n < R) {
-            BGS_CUDA(bgs::launch_iota(p->iota_n, R, gidx, s), "record indices");
-            p->host_launches += 1;
-            cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-            if (cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone) p->iota_n = R;
-        }
         size_t tmp = 0;
         BGS_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tmp, k0, k1, gidx, order, (int64_t)N, 0, 32, s),
                  "view depth sort (size)");
         // the views' sorts are independent: fork them over the side streams (a fork-join of
         // events, which a graph capture records as such) and join before the binning
         // (one view: no fork, everything on the caller's stream)
-        const int NS = std::min<int>(V, kSortStreams);
+        // (eight streams for views of fewer than 2M Gaussians, whose counting passes leave most of
+        // the chip idle: 16 views of 500k 2.45 -> 2.17 ms; four for larger ones, which fill it: the
+        // 9-view 4M step 12.52 ms with four, 12.57 with eight)
+        const int NS = std::min<int>(V, N < (2ll << 20) ? kSortStreams : kSortStreams / 2);
         auto stream_of = [&](int i) { return NS > 1 ? p->sort_stream[i] : s; };
         for (int i = 0; i < NS; ++i) BGS_TRY(ensure(p, p->sort_tmp[i], tmp, s, "sort_tmp"));
         if (NS > 1) {
@@ -1339,27 +1371,30 @@ int bgs_bin_and_sort_batched(bgs_plan *p, int32_t V, const bgs_view *views, int6
             cudaStream_t si = stream_of(i);
             BinView bv;
             BGS_TRY(bin_view_a(p, i, v, N, order + (size_t)v * N, means2D, radii, conic_opacity, Ws[v], Hs[v], tw, th,
-                               bv, si));
+                               V == 1, sync ? kSyncCapacity : capacity, ranges + 2ull * vt.tile_base[v], bv, si));
             if (NS > 1) {
+                // view v's lists need the counts of views 0..v-1: its event waits for the view
+                // before it, so that one wait stands for all
+                if (v > 0) BGS_CUDA(cudaStreamWaitEvent(si, p->view_done[v - 1], 0), "earlier view counts");
                 BGS_CUDA(cudaEventRecord(p->view_done[v], si), "view count done");
-                for (int u = 0; u < v; ++u)
-                    if (u % NS != i) BGS_CUDA(cudaStreamWaitEvent(si, p->view_done[u], 0), "earlier view counts");
             }
-            BGS_TRY(bin_view_b(p, i, v, N, bv, Ws[v], Hs[v], tw, th, point_list, capacity,
-                               ranges + 2ull * vt.tile_base[v], si));
+            BGS_TRY(bin_view_b(p, i, v, N, bv, Ws[v], Hs[v], tw, th, point_list, capacity, si));
         }
         for (int i = 0; i < NS && NS > 1; ++i) {
             BGS_CUDA(cudaEventRecord(p->sort_join[i], p->sort_stream[i]), "binning join");
             BGS_CUDA(cudaStreamWaitEvent(s, p->sort_join[i], 0), "binning join wait");
         }
-        BGS_CUDA(bgs::launch_bin_finish(V, sync ? (1ll << 62) : capacity, p->ctrl, s), "bin_finish");
-        p->host_launches += 1;
+        if (V > 1) {
+            BGS_CUDA(bgs::launch_bin_finish(V, sync ? kSyncCapacity : capacity, p->ctrl,
+                                            sync ? p->host_k_dev : nullptr, s), "bin_finish");
+            p->host_launches += 1;
+        }
     }
     if (!sync) return BGS_OK;
     unsigned long long K = 0;
     if (R > 0) {
-        BGS_CUDA(cudaMemcpyAsync(&K, &p->ctrl->num_entries, sizeof K, cudaMemcpyDeviceToHost, s), "read K");
         BGS_CUDA(cudaStreamSynchronize(s), "sync K");
+        K = *(volatile unsigned long long *)p->host_k;
     }
     if (needed) *needed = (int64_t)K;
     if ((long long)K > capacity || (long long)K > BGS_MAX_ENTRIES)

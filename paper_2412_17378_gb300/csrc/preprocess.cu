@@ -416,11 +416,10 @@ cudaError_t launch_iota(long long lo, long long hi, uint32_t *idx, cudaStream_t 
 // keeping the depth order.  This moves the multi-pass work from K 12-byte records over
 // 45 key bits to K 6- or 8-byte records over the tile bits only.
 
-// Entry count (rectangle area) and depth sort key of each Gaussian.
+// Entry count (rectangle area) of each Gaussian.
 __global__ void __launch_bounds__(256) k_touched(long long N, const float2 *__restrict__ means2D,
-                                                 const int *__restrict__ radii, const float *__restrict__ depths,
-                                                 int tw, int th, int tx, int ty, uint32_t *__restrict__ touched,
-                                                 uint32_t *__restrict__ dkey, uint32_t *__restrict__ idx) {
+                                                 const int *__restrict__ radii, int tw, int th, int tx, int ty,
+                                                 uint32_t *__restrict__ touched) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const int r = radii[i];
@@ -432,16 +431,14 @@ __global__ void __launch_bounds__(256) k_touched(long long N, const float2 *__re
         if (x1 > x0 && y1 > y0) c = (uint32_t)((x1 - x0) * (y1 - y0));
     }
     touched[i] = c;
-    dkey[i] = __float_as_uint(depths[i]);
-    idx[i] = (uint32_t)i;
 }
 
-cudaError_t launch_touched(long long N, const float *means2D, const int *radii, const float *depths, int W, int H,
-                           int tile_w, int tile_h, uint32_t *touched, uint32_t *dkey, uint32_t *idx, cudaStream_t s) {
+cudaError_t launch_touched(long long N, const float *means2D, const int *radii, int W, int H, int tile_w, int tile_h,
+                           uint32_t *touched, cudaStream_t s) {
     if (N == 0) return cudaSuccess;
     const int tx = (W + tile_w - 1) / tile_w, ty = (H + tile_h - 1) / tile_h;
-    k_touched<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(N, reinterpret_cast<const float2 *>(means2D), radii, depths,
-                                                          tile_w, tile_h, tx, ty, touched, dkey, idx);
+    k_touched<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(N, reinterpret_cast<const float2 *>(means2D), radii, tile_w,
+                                                          tile_h, tx, ty, touched);
     return cudaGetLastError();
 }
 
