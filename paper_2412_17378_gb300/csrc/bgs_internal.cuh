@@ -47,6 +47,7 @@ struct DevCtrl {
     unsigned long long view_k[kMaxViews];
     unsigned long long view_base[kMaxViews];
     unsigned int bin_done[kMaxViews];  // column blocks done (returns to zero)
+    unsigned int bin_head[kMaxViews];  // the scatter's queue cursor
 };
 
 // End of a persistent pass, per warp (lane 0), for a block of `warps_per_block` warps whose
@@ -409,12 +410,14 @@ cudaError_t launch_bin_stopped(int B1, int tx, int ty, const uint16_t *D, uint32
 // and, from the view's first point_list slot on, its range; the scatter's items per tile group
 // (with truncation); for a call's only view the call's entry count, also to host_k (nullable,
 // mapped host memory), with the overflow check against capacity.
+constexpr int kScatterBlocks = 32;  // single-warp blocks of the scatter per SM
 struct BinTiles {
     int T, tx, ty, B, nC, v;
     uint32_t *total, *start;
     uint2 *ranges;
     const uint32_t *bsat;  // nullable: complete lists
-    uint32_t *item_start;
+    uint32_t *item_start;  // [4 nC + 1], see open_items
+    int warps;             // resident warps of the scatter
     bool only;             // the call's only view
     long long capacity;
     unsigned long long *host_k;
@@ -435,7 +438,7 @@ cudaError_t launch_bin_open(const BinTiles &bt, cudaStream_t s);
 cudaError_t launch_bin_scatter(long long N, int G, int B, int W32, const uint4 *rect, int W, int H, int tw, int th,
                                const uint32_t *Hm, const uint32_t *start, const uint32_t *masks, uint32_t *point_list,
                                long long capacity, const uint32_t *bsat, const uint32_t *item_start, int num_sms,
-                               int v, const DevCtrl *ctrl, cudaStream_t s);
+                               int v, DevCtrl *ctrl, cudaStream_t s);
 // num_entries = bin_base = the sum of the V views' counts, also to host_k (nullable); raises
 // BGS_CHECK_OVERFLOW past capacity or BGS_MAX_ENTRIES
 cudaError_t launch_bin_finish(int V, long long capacity, DevCtrl *ctrl, unsigned long long *host_k, cudaStream_t s);

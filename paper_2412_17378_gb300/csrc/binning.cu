@@ -26,8 +26,8 @@
 //                      tile the rectangle covers (and whose list was not cut before b)
 //                      appends the index.  A lane stages
 //                      its appends in a 16-word ring in shared memory and writes each
-//                      completed 32-byte sector of its run with two 16-byte stores, so the
-//                      point list is written in whole sectors (not one word per request).
+//                      completed 32-byte sector of its run with one store, so the point list
+//                      is written in whole sectors (not one word per request).
 // The result is the stable (depth, index) order per tile.  Traffic is O(B T + K) words
 // instead of the ~26 bytes per entry of a two-pass radix sort of (tile, index) pairs.
 #include <algorithm>
@@ -436,8 +436,9 @@ __device__ __forceinline__ void publish_count(unsigned long long k, long long ca
 }
 
 // Exclusive scan of the tile totals by the 32 warps of one block, each over a run of tiles read 32
-// at a time: start[t], the 64-bit count of the view and, for a call's only view, its ranges.
-__device__ __forceinline__ void scan_tiles(const BinTiles &bt, int tid) {
+// at a time: start[t], the 64-bit count of the view (returned) and, for a call's only view, its
+// ranges.
+__device__ __forceinline__ unsigned long long scan_tiles(const BinTiles &bt, int tid) {
     __shared__ unsigned long long part[32];
     const int lane = tid & 31, warp = tid >> 5;
     const int per = ((bt.T + 1023) / 1024) * 32, t0 = min(bt.T, warp * per), t1 = min(bt.T, t0 + per);
@@ -477,28 +478,81 @@ __device__ __forceinline__ void scan_tiles(const BinTiles &bt, int tid) {
             publish_count(K, bt.capacity, bt.ctrl, bt.host_k);
         }
     }
+    return K;
 }
 
-// Work items of the scatter: the (depth block b, tile group C) pairs with b at most the last
-// block any tile of C keeps, numbered C-major.  By the 1024 threads of one block, a lane per
-// tile of a group while its last block is found: item_start[C] = exclusive prefix of min(B, max
-// over C's tiles of b_sat + 1), and item_start[nC] = the item count.
-__device__ __forceinline__ void open_items(const BinTiles &bt, int tid) {
-    __shared__ uint32_t part[32];
+// Work items of the scatter of truncated lists: per tile group C the depth blocks up to the last
+// one any tile of C keeps, in runs of r consecutive blocks: about `target` entries an item.  A
+// sparse group's blocks hold a few entries each, and an item's fixed cost (its search, loads,
+// first and last sectors: about 600 instructions) outweighed them; a dense group's blocks stay
+// items of their own.  (16 views of 500k 2087 -> 2020 us, the 9-view 4M step 12.15 -> 12.01 ms.
+// Complete lists, whose groups are denser, take one block of one group each: 352 us for 1M at
+// 1080p, 358 with these items.)  target gives every resident warp about eight items, within
+// 128 .. 2048.  The groups come densest first (by the power of two of their entries per block):
+// a block that all of its 2048 Gaussians hit is 40 us of one warp's work, and one that starts
+// late is the kernel's tail.  By the 1024 threads of one block, a lane per tile of a group while
+// its last block and entries are found.  Written, for the k-th group: start[k] = exclusive
+// prefix of the groups' item counts (start[nC]: all of them), then C[k], r[k] and the first
+// block past its last.
+constexpr int kSortGroups = 1536;  // (a 3840 x 2160 view has 1020); grids of more keep their order
+
+__device__ __forceinline__ void open_items(const BinTiles &bt, int tid, unsigned long long K) {
+    __shared__ uint32_t part[32], place[33];
+    __shared__ uint32_t s_r[kSortGroups], s_n[kSortGroups];
+    __shared__ unsigned char s_cls[kSortGroups];
     const int lane = tid & 31, warp = tid >> 5;
     const int nC = bt.nC, ncx = (bt.tx + kCbW - 1) / kCbW;
+    uint32_t *start = bt.item_start, *group = start + nC + 1, *run_of = group + nC, *end_of = run_of + nC;
+    const uint32_t target = (uint32_t)min(2048ull, max(128ull, K / (8ull * bt.warps)));
+    const bool sorted = nC <= kSortGroups;
+    if (tid < 33) place[tid] = 0u;
+    __syncthreads();
 #pragma unroll 4
     for (int C = warp; C < nC; C += 32) {
         const int x = (C % ncx) * kCbW + lane % kCbW, y = (C / ncx) * kCbH + lane / kCbW;
-        const uint32_t last = x < bt.tx && y < bt.ty ? __ldcg(bt.bsat + (size_t)y * bt.tx + x) : 0u;
+        const bool in = x < bt.tx && y < bt.ty;
+        const size_t t = (size_t)y * bt.tx + x;
+        const uint32_t last = in ? __ldcg(bt.bsat + t) : 0u, ent = in ? __ldcg(bt.total + t) : 0u;
         const uint32_t n = min((uint32_t)bt.B, __reduce_max_sync(0xffffffffu, last) + 1u);
-        if (lane == 0) bt.item_start[C] = n;  // the count, turned into the offset below
+        const uint32_t E = __reduce_add_sync(0xffffffffu, min(ent, 1u << 26));
+        if (lane == 0) {
+            const float each = (float)E / (float)n;  // entries per block
+            const uint32_t r = E ? min(n, max(1u, (uint32_t)((float)target / each))) : n;
+            if (sorted) {
+                const uint32_t cls = E ? (uint32_t)__clz((uint32_t)each + 1u) : 32u;
+                s_r[C] = r, s_n[C] = E ? n : 0u, s_cls[C] = (unsigned char)cls;
+                atomicAdd(&place[cls], 1u);
+            } else {
+                group[C] = (uint32_t)C, run_of[C] = r, end_of[C] = n;
+                start[C] = E ? (n + r - 1u) / r : 0u;  // the count, turned into the offset below
+            }
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {  // the classes' places
+        const uint32_t u = place[lane];
+        uint32_t incl = u;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t w = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += w;
+        }
+        place[lane] = incl - u;
+        if (lane == 31) place[32] = incl;
+        if (lane == 0) bt.ctrl->bin_head[bt.v] = 0u;
+    }
+    __syncthreads();
+    for (int C = tid; sorted && C < nC; C += 1024) {  // (the order within a class is any)
+        const uint32_t k = atomicAdd(&place[s_cls[C]], 1u), r = s_r[C], n = s_n[C];
+        group[k] = (uint32_t)C;
+        run_of[k] = r;
+        end_of[k] = n;
+        start[k] = (n + r - 1u) / r;
     }
     __syncthreads();
     uint32_t run = 0;
-    for (int c0 = 0; c0 < nC; c0 += 1024) {  // 1024 groups at a time (a 3840 x 2160 view has 1020)
-        const int C = c0 + tid;
-        const uint32_t n = C < nC ? bt.item_start[C] : 0u;
+    for (int c0 = 0; c0 < nC; c0 += 1024) {
+        const int k = c0 + tid;
+        const uint32_t n = k < nC ? start[k] : 0u;
         uint32_t incl = n;
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
@@ -512,10 +566,10 @@ __device__ __forceinline__ void open_items(const BinTiles &bt, int tid) {
             if (w < warp) base += u;
             run += u;
         }
-        if (C < nC) bt.item_start[C] = base + incl - n;
+        if (k < nC) start[k] = base + incl - n;
         __syncthreads();
     }
-    if (tid == 0) bt.item_start[nC] = run;
+    if (tid == 0) start[nC] = run;
 }
 
 // Block (32 tiles) x (32 row groups): per column t, exclusive prefix over b in place, and
@@ -528,7 +582,7 @@ __device__ __forceinline__ void open_items(const BinTiles &bt, int tid) {
 // each, on one block or a few).  With the key pass and the copies of the count gone as well, a
 // 256 x 256 frame of 10k Gaussians takes 232 instead of 270 us, the lists of 1M at 1080p 378
 // instead of 420.
-__global__ void __launch_bounds__(1024) k_bin_colscan(uint32_t *__restrict__ H, const uint16_t *__restrict__ D,
+__global__ void __launch_bounds__(1024, 2) k_bin_colscan(uint32_t *__restrict__ H, const uint16_t *__restrict__ D,
                                                       uint32_t thr, const BinTiles bt, uint32_t *__restrict__ bsat) {
     __shared__ bool s_last;
     const int B = bt.B, T = bt.T;
@@ -611,8 +665,8 @@ __global__ void __launch_bounds__(1024) k_bin_colscan(uint32_t *__restrict__ H, 
     if (!s_last) return;
     __threadfence();
     if (tid == 0) bt.ctrl->bin_done[bt.v] = 0u;
-    scan_tiles(bt, tid);
-    if (bt.only && bt.bsat) open_items(bt, tid);
+    const unsigned long long K = scan_tiles(bt, tid);
+    if (bt.only && bt.bsat) open_items(bt, tid, K);
 }
 
 // A view of several, one block: ranges[t] = base + [start[t], start[t] + n[t]) ((0,0) for an
@@ -626,7 +680,7 @@ __global__ void __launch_bounds__(1024) k_bin_open(const BinTiles bt) {
         const uint32_t a = base + bt.start[t], n = bt.total[t];
         bt.ranges[t] = n ? make_uint2(a, a + n) : make_uint2(0u, 0u);
     }
-    if (bt.bsat) open_items(bt, threadIdx.x);
+    if (bt.bsat) open_items(bt, threadIdx.x, bt.ctrl->view_k[bt.v]);
 }
 
 // The call's entry count over its V views.
@@ -646,9 +700,11 @@ __device__ __forceinline__ void flush_sector(const uint32_t *ring_s, int lane, u
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = src[32 * j];
     if (vec_ok && done >= run0 && done + 8u <= capacity) {
-        uint4 *dst = reinterpret_cast<uint4 *>(point_list + done);  // 32-byte aligned
-        dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
-        dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
+        // one 32-byte store (32-byte aligned): each lane's goes to a line of its own, and the stores
+        // of two halves took the first-level cache twice the passes
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(point_list + done), "r"(v[0]),
+                     "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                     : "memory");
     } else {
 #pragma unroll
         for (int j = 0; j < 8; ++j)
@@ -660,59 +716,66 @@ __device__ __forceinline__ void flush_sector(const uint32_t *ring_s, int lane, u
 // Single-warp blocks: a block's shared memory is released as soon as its warp is done
 // (blocks of several warps hold it until the slowest one finishes, and reached fewer
 // resident warps).
-// With truncated lists (bsat given) the blocks stride over the work items of k_bin_items,
-// item -> (C, b); with complete lists every (b, C) is an item and block i takes item i
-// (C = i / B, b = i % B) once.  Item (b, C): one warp, lane l owns tile l of C; lanes whose
-// list ends before b append nothing.
+// With truncated lists (bsat given) the warps take the work items of open_items in order from a
+// queue: item -> (C, blocks [b0, b1)); with complete lists block i takes the item (C = i / B,
+// block i % B).  Lane l owns tile l of C; lanes whose list ends before a block append nothing
+// from there on.
 __global__ void __launch_bounds__(32) k_bin_scatter(uint32_t G, int W32, const uint4 *__restrict__ rect, int tx, int ty,
                                                     const uint32_t *__restrict__ H, const uint32_t *__restrict__ start,
                                                     const uint32_t *__restrict__ masks,
                                                     uint32_t *__restrict__ point_list, uint32_t capacity, int vec_ok,
                                                     const uint32_t *__restrict__ bsat,
                                                     const uint32_t *__restrict__ item_start, int nC, int B,
-                                                    int v, const DevCtrl *ctrl) {
+                                                    int v, DevCtrl *ctrl) {
     // per flagged Gaussian of the pass: (lanes whose tile its rectangle covers, Gaussian
     // index), .y holding its sorted position until the hit is known; and the lanes' 16-word
-    // output rings, slot-major.  7 KB of shared memory a block in all, so that 32 blocks
+    // output rings, slot-major.  6 KB of shared memory a block in all, so that 32 blocks
     // (the per-SM block limit) fit an SM.
     __shared__ uint2 hit_s[512];
     __shared__ uint32_t ring_s[16 * 32];
     const int lane = threadIdx.x;
     const int ncx = (tx + kCbW - 1) / kCbW;
     const bool listed = bsat != nullptr;
-    const uint32_t n_items = listed ? item_start[nC] : (uint32_t)B * (uint32_t)nC;
+    const uint32_t n_items = listed ? item_start[nC] : 0u;
+    const uint32_t *group = item_start + nC + 1, *run_of = group + nC, *end_of = run_of + nC;
     const uint32_t base = (uint32_t)ctrl->view_base[v];
     uint32_t *ring = ring_s + lane;
-    for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
-        int C, b;
+    do {
+        int C;
+        uint32_t b0, b1;
         if (listed) {
-            int lo = 0, hi = nC - 1;  // C: the last group with item_start[C] <= it
+            uint32_t it = 0;
+            if (lane == 0) it = atomicAdd(&ctrl->bin_head[v], 1u);
+            it = __shfl_sync(0xffffffffu, it, 0);
+            if (it >= n_items) break;
+            int lo = 0, hi = nC - 1;  // the last group with start <= it
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
                 if (item_start[mid] <= it) lo = mid;
                 else hi = mid - 1;
             }
-            C = lo;
-            b = (int)(it - item_start[C]);
+            C = (int)group[lo];
+            b0 = (it - item_start[lo]) * run_of[lo];
+            b1 = min(end_of[lo], b0 + run_of[lo]);
         } else {
-            C = (int)(it / (uint32_t)B);
-            b = (int)(it % (uint32_t)B);
+            C = (int)(blockIdx.x / (uint32_t)B);
+            b0 = blockIdx.x % (uint32_t)B;
+            b1 = b0 + 1u;
         }
         const int gx0 = (C % ncx) * kCbW, gy0 = (C / ncx) * kCbH;
         const int ltx = gx0 + (lane % kCbW), lty = gy0 + (lane / kCbW);
         const size_t t = (size_t)lty * tx + ltx;
-        // a lane whose tile's list was cut before block b appends nothing
-        const bool own = ltx < tx && lty < ty && (bsat == nullptr || (uint32_t)b <= bsat[t]);
-        const unsigned own_mask = __ballot_sync(0xffffffffu, own);
+        // one past the last block the lane's tile keeps
+        const uint32_t keep_to = ltx < tx && lty < ty ? (bsat ? bsat[t] + 1u : 0xffffffffu) : 0u;
+        unsigned own_mask = __ballot_sync(0xffffffffu, b0 < keep_to);
         if (own_mask == 0u) continue;
-        uint32_t pos = own ? base + start[t] + H[(size_t)b * tx * ty + t] : 0u;
+        uint32_t pos = b0 < keep_to ? base + start[t] + H[(size_t)b0 * tx * ty + t] : 0u;
         const uint32_t run0 = pos;
         uint32_t done = pos & ~7u;  // positions below done are written (or precede the run)
-        const uint32_t *mk = masks + ((size_t)b * nC + C) * W32;
-        const uint32_t s0 = (uint32_t)b * G;
-        // The flagged positions of the item's mask words, 16 words (512 Gaussians) a pass,
-        // gathered in depth order into hit_s across passes and visited in batches of up to 512
-        // hits: one round of rectangle gathers serves all passes of a sparse item.
+        // The flagged positions of the blocks' mask words, 64 words (2048 Gaussians) a pass, two to a
+        // lane, gathered in depth order into hit_s across passes and blocks and visited in batches
+        // of up to 512 hits: one scan serves 64 words, and one round of rectangle gathers all the
+        // passes of a sparse item.
         auto visit = [&](int total) {
             // per flagged Gaussian: the lanes whose tile its rectangle covers (a nonempty
             // rectangle meeting the group: the masks flag no other), among the lanes whose
@@ -771,38 +834,74 @@ __global__ void __launch_bounds__(32) k_bin_scatter(uint32_t G, int W32, const u
             __syncwarp();
         };
         int acc = 0;  // hits gathered in hit_s[0, acc)
-        uint32_t next = lane < 16 ? mk[lane] : 0u;
-        for (int wb = 0; wb < W32; wb += 16) {
-            uint32_t word = next;
-            next = (lane < 16 && wb + 16 < W32) ? mk[wb + 16 + lane] : 0u;  // the next pass's words, early
-            const uint32_t cnt = (uint32_t)__popc(word);
-            uint32_t incl = cnt;
-            for (int o = 1; o < 16; o <<= 1) {
-                const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+        bool last_of = false;  // the hits gathered after this pass belong to fewer tiles
+        unsigned own_next = own_mask;
+        // (the word arrays are 16-word aligned: W32 is a multiple of 16)
+        const size_t stride = (size_t)nC * W32;  // from a block's words to the next's
+        const uint32_t *mk = masks + b0 * stride + (size_t)C * W32;
+        auto words = [&](const uint32_t *m, int wb) {
+            return wb + 2 * lane < W32 ? *reinterpret_cast<const uint2 *>(m + wb + 2 * lane) : make_uint2(0u, 0u);
+        };
+        uint2 next = words(mk, 0);
+        uint32_t b = b0;
+        for (int wb = 0; b < b1;) {
+            uint2 w = next;
+            const uint32_t s0 = b * G + 32u * (uint32_t)wb;
+            // the next pass's words, early
+            wb += 64;
+            if (wb >= W32) wb = 0, ++b, mk += stride;
+            if (b < b1) next = words(mk, wb);
+            if (wb == 0) {  // the last pass of its block: does a tile's list end with it?
+                const unsigned still = __ballot_sync(0xffffffffu, b < keep_to);
+                last_of = still != own_mask;
+                own_next = still;
+            }
+            const int cnt = __popc(w.x) + __popc(w.y);
+            int incl = cnt;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += u;
             }
-            const int total = (int)__shfl_sync(0xffffffffu, incl, 15);
-            if (total == 0) continue;
-            if (acc + total > 512) {
-                visit(acc);
+            const int total = __shfl_sync(0xffffffffu, incl, 31);
+            // all lanes' words at once, or, past 512 hits, 16 words (8 lanes, at most 512) at a time
+            const int step = total <= 512 ? 32 : 8;
+            for (int l0 = 0; total > 0 && l0 < 32; l0 += step) {
+                const int before = l0 > 0 ? __shfl_sync(0xffffffffu, incl, l0 - 1) : 0;
+                const int part = __shfl_sync(0xffffffffu, incl, l0 + step - 1) - before;
+                if (acc + part > 512) {
+                    visit(acc);
+                    acc = 0;
+                }
+                // compact the flagged positions in depth order (word by word, bit by bit)
+                if (lane >= l0 && lane < l0 + step) {
+                    int off = acc + incl - cnt - before;
+                    const uint32_t p0 = s0 + 64u * (uint32_t)lane;
+                    while (w.x) {
+                        hit_s[off++].y = p0 + (uint32_t)(__ffs(w.x) - 1);
+                        w.x &= w.x - 1u;
+                    }
+                    while (w.y) {
+                        hit_s[off++].y = p0 + 32u + (uint32_t)(__ffs(w.y) - 1);
+                        w.y &= w.y - 1u;
+                    }
+                }
+                __syncwarp();
+                acc += part;
+            }
+            if (last_of) {
+                if (acc) visit(acc);
                 acc = 0;
+                own_mask = own_next;
+                last_of = false;
+                if (own_mask == 0u) break;
             }
-            // compact the flagged positions in depth order (word by word, bit by bit)
-            uint32_t off = (uint32_t)acc + incl - cnt;
-            while (word) {
-                const int bit = __ffs(word) - 1;
-                word &= word - 1u;
-                hit_s[off++].y = s0 + 32u * (uint32_t)(wb + lane) + (uint32_t)bit;
-            }
-            __syncwarp();
-            acc += total;
         }
         if (acc) visit(acc);
         // the last, partial sector
         for (uint32_t p = done; p < pos; ++p)
             if (p >= run0 && p < capacity) point_list[p] = ring[(p & 15u) << 5];
         __syncwarp();
-    }
+    } while (listed);
 }
 
 size_t bin_count_smem(int tx, int ty) {
@@ -964,7 +1063,7 @@ cudaError_t launch_bin_finish(int V, long long capacity, DevCtrl *ctrl, unsigned
 cudaError_t launch_bin_scatter(long long N, int G, int B, int W32, const uint4 *rect, int W, int H, int tw, int th,
                                const uint32_t *Hm, const uint32_t *start, const uint32_t *masks, uint32_t *point_list,
                                long long capacity, const uint32_t *bsat, const uint32_t *item_start, int num_sms,
-                               int v, const DevCtrl *ctrl, cudaStream_t s) {
+                               int v, DevCtrl *ctrl, cudaStream_t s) {
     (void)N;
     const int tx = (W + tw - 1) / tw, ty = (H + th - 1) / th;
     const int nC = bin_mask_groups(tx, ty);
@@ -972,11 +1071,9 @@ cudaError_t launch_bin_scatter(long long N, int G, int B, int W32, const uint4 *
     const uint32_t cap = capacity > BGS_MAX_ENTRIES ? (uint32_t)BGS_MAX_ENTRIES : (uint32_t)capacity;
     const int vec_ok = (reinterpret_cast<uintptr_t>(point_list) & 31u) == 0u;
     // truncated lists: a persistent grid (32 single-warp blocks per SM, the per-SM block limit)
-    // over the open items; complete lists: one block per (b, C), scheduled by the hardware
+    // over the items; complete lists: one block per (b, C), scheduled by the hardware
     long long grid = (long long)B * nC;
-    if (bsat) {
-        grid = std::min<long long>((long long)num_sms * 32, grid);
-    }
+    if (bsat) grid = std::min<long long>((long long)num_sms * kScatterBlocks, grid);
     k_bin_scatter<<<(unsigned)std::max<long long>(1, grid), 32, 0, s>>>((uint32_t)G, W32, rect, tx, ty, Hm, start,
                                                                          masks, point_list, cap, vec_ok, bsat,
                                                                          item_start, nC, B, v, ctrl);

@@ -83,12 +83,11 @@ struct bgs_plan {
     unsigned long long host_launches = 0;
     // binning
     Buf touched, touched_sorted, dkey_sorted, gidx, order, offsets, keys_in, keys_out, vals_in, cub_tmp;
-    // counting-sort binning, one buffer set per concurrent view (stream slot): tile histogram,
-    // totals, starts, packed rectangles, masks; list truncation (credits, last block per
-    // tile); the scatter's work items per tile group
+    // counting-sort binning, one set per concurrent view (stream slot): all of a view's scratch in
+    // one allocation (its parts are laid out by bin_sizes), and the per-tile sums of the
+    // stopped-tile passes, zero between passes whatever their grid (each pass clears what it read)
     struct BinSlot {
-        Buf h, total, start, rect, mask, credit, sat, items, stopped;
-        Buf stopped_sum;  // zero between passes, whatever their grid (each pass clears what it read)
+        Buf arena, stopped_sum;
     } bin_slot[kSortStreams];
     cudaEvent_t view_done[bgs::kMaxViews] = {};  // a view's entry count is known
     int smem_optin = 0;
@@ -422,9 +421,7 @@ int bgs_plan_destroy(bgs_plan *p) {
     for (cudaEvent_t e : p->view_done)
         if (e) cudaEventDestroy(e);
     for (auto &sl : p->bin_slot) {
-        Buf *sb[] = {&sl.h, &sl.total, &sl.start, &sl.rect, &sl.mask, &sl.credit, &sl.sat, &sl.items, &sl.stopped,
-                     &sl.stopped_sum};
-        for (Buf *b : sb)
+        for (Buf *b : {&sl.arena, &sl.stopped_sum})
             if (b->p) cudaFree(b->p);
     }
     Buf *bufs[] = {&p->gw_exoff, &p->gw_ent, &p->gw_done, &p->gw_sum, &p->gw_tile, &p->tile_cost, &p->vkey_sorted, &p->touched, &p->touched_sorted,
@@ -693,27 +690,36 @@ constexpr long long kBinPassDiv[2] = {8, 2};
 constexpr long long kSyncCapacity = 1ll << 62;
 
 struct BinView {
-    int tiles_x, tiles_y;
+    int tiles_x, tiles_y, passes;
     long long T, G, B, W32, nC;
     bool trunc;
+    // byte offsets of the scratch's parts: tile histogram, totals, starts, packed rectangles,
+    // masks, the scatter's items; credits, last block per tile (trunc); stopped-tile prefix
+    // (passes > 1); then its size
+    size_t h, total, start, rect, mask, items, credit, sat, stopped, bytes;
     bgs::BinTiles tiles;
 };
 
-int bin_view_a(bgs_plan *p, int slot, int v, long long n, const uint32_t *order, const float *means2D,
-               const int32_t *radii, const float *conic_opacity, int W, int H, int tw, int th, bool only,
-               long long capacity, uint32_t *ranges, BinView &bv, cudaStream_t s) {
-    bgs_plan::BinSlot &sl = p->bin_slot[slot];
+// The blocking of a view of n Gaussians and the layout of its scratch.
+int bin_sizes(const bgs_plan *p, long long n, bool conics, int W, int H, int tw, int th, BinView &bv) {
     bv.tiles_x = (W + tw - 1) / tw;
     bv.tiles_y = (H + th - 1) / th;
     const long long T = bv.T = (long long)bv.tiles_x * bv.tiles_y;
-    const size_t smem = bgs::bin_count_smem(bv.tiles_x, bv.tiles_y);
-    if (smem > (size_t)p->smem_optin) return fail(BGS_ERR_INVALID, "tile grid too large for counting-sort binning");
+    if (bgs::bin_count_smem(bv.tiles_x, bv.tiles_y) > (size_t)p->smem_optin)
+        return fail(BGS_ERR_INVALID, "tile grid too large for counting-sort binning");
+    // list truncation: per-block credits toward the certificate that a tile's pixels have all
+    // stopped (needs the conics, and the credit counters of one block in shared memory)
+    bv.trunc = conics && bgs::bin_credit_smem(bv.tiles_x, bv.tiles_y) <= (size_t)p->smem_optin;
     // G: a multiple of 32.  Automatic: at least 2048, about 4 counting blocks per SM (fewer,
     // longer blocks keep the scatter's per-(block, tile group) overhead down), and large
     // enough that B T stays below 2^24
     long long G = p->desc.bin_block;
     if (G <= 0) {
-        G = std::max<long long>(2048, (n + 4ll * p->num_sms - 1) / (4ll * std::max(1, p->num_sms)));
+        // (few Gaussians with complete lists: smaller blocks, so that more than a handful of warps
+        // count and scatter: a 256 x 256 frame of 10k 226 -> 204 us; truncated lists are cut at a
+        // block's end, which stays where it was)
+        const long long least = conics || n >= (1 << 18) ? 2048 : (n >= (1 << 16) ? 1024 : 512);
+        G = std::max<long long>(least, (n + 4ll * p->num_sms - 1) / (4ll * std::max(1, p->num_sms)));
         G = std::max<long long>(G, (n * T + (1ll << 24) - 1) >> 24);
     }
     G = bv.G = (G + 31) & ~31ll;
@@ -721,50 +727,66 @@ int bin_view_a(bgs_plan *p, int slot, int v, long long n, const uint32_t *order,
     const long long W32 = bv.W32 = ((G + 511) / 512) * 16;  // mask words per (block, tile group)
     const long long nC = bv.nC = bgs::bin_mask_groups(bv.tiles_x, bv.tiles_y);
     if (B * T >= (1ll << 31) || B * nC * W32 >= (1ll << 40)) return fail(BGS_ERR_INVALID, "tile histogram too large");
-    BGS_TRY(ensure(p, sl.h, sizeof(uint32_t) * B * T, s, "bin_h"));
-    BGS_TRY(ensure(p, sl.total, sizeof(uint32_t) * T, s, "bin_total"));
-    BGS_TRY(ensure(p, sl.start, sizeof(uint32_t) * T, s, "bin_start"));
-    BGS_TRY(ensure(p, sl.rect, sizeof(uint4) * n, s, "bin_rect"));
-    BGS_TRY(ensure(p, sl.mask, sizeof(uint32_t) * B * nC * W32, s, "bin_mask"));
-    uint32_t *Hm = (uint32_t *)sl.h.p, *tot = (uint32_t *)sl.total.p, *start = (uint32_t *)sl.start.p;
-    uint4 *rect = (uint4 *)sl.rect.p;
-    if (smem > 48 * 1024) BGS_CUDA(bgs::setup_bin_kernels(bv.tiles_x, bv.tiles_y), "bin smem attribute");
-    // list truncation: per-block credits toward the certificate that a tile's pixels have all
-    // stopped (needs the conics, and the credit counters of one block in shared memory)
-    bv.trunc = conic_opacity && bgs::bin_credit_smem(bv.tiles_x, bv.tiles_y) <= (size_t)p->smem_optin;
-    uint16_t *credit = nullptr;
-    uint32_t *bsat = nullptr;
-    if (bv.trunc) {
-        BGS_TRY(ensure(p, sl.credit, sizeof(uint16_t) * B * T, s, "bin_credit"));
-        BGS_TRY(ensure(p, sl.sat, sizeof(uint32_t) * T, s, "bin_sat"));
-        credit = (uint16_t *)sl.credit.p;
-        bsat = (uint32_t *)sl.sat.p;
-    }
+    bv.passes = bv.trunc && B >= 32 ? 3 : 1;
+    size_t at = 0;
+    auto part = [&](size_t bytes) {
+        const size_t o = at;
+        at += (bytes + 255) & ~(size_t)255;
+        return o;
+    };
+    bv.h = part(sizeof(uint32_t) * B * T);
+    bv.total = part(sizeof(uint32_t) * T);
+    bv.start = part(sizeof(uint32_t) * T);
+    bv.rect = part(sizeof(uint4) * n);
+    bv.mask = part(sizeof(uint32_t) * B * nC * W32);
+    bv.items = part(sizeof(uint32_t) * (4 * nC + 1));
+    bv.credit = part(bv.trunc ? sizeof(uint16_t) * B * T : 0);
+    bv.sat = part(bv.trunc ? sizeof(uint32_t) * T : 0);
+    bv.stopped = part(bv.passes > 1 ? sizeof(int) * (size_t)(bv.tiles_x + 1) * (bv.tiles_y + 1) : 0);
+    bv.bytes = at;
+    return BGS_OK;
+}
+
+// The scratch of a slot for views of at most these sizes.
+int ensure_bin_slot(bgs_plan *p, int slot, size_t bytes, long long tiles, cudaStream_t s) {
+    bgs_plan::BinSlot &sl = p->bin_slot[slot];
+    BGS_TRY(ensure(p, sl.arena, bytes, s, "binning"));
+    if (tiles == 0) return BGS_OK;
+    const size_t before = sl.stopped_sum.bytes;
+    BGS_TRY(ensure(p, sl.stopped_sum, sizeof(uint32_t) * tiles, s, "bin_stopped_sum"));
+    if (sl.stopped_sum.bytes != before)
+        BGS_CUDA(cudaMemsetAsync(sl.stopped_sum.p, 0, sl.stopped_sum.bytes, s), "clear bin_stopped_sum");
+    return BGS_OK;
+}
+
+// bv: as bin_sizes left it, its slot's scratch large enough.
+int bin_view_a(bgs_plan *p, int slot, int v, long long n, const uint32_t *order, const float *means2D,
+               const int32_t *radii, const float *conic_opacity, int W, int H, int tw, int th, bool only,
+               long long capacity, uint32_t *ranges, BinView &bv, cudaStream_t s) {
+    char *base = (char *)p->bin_slot[slot].arena.p;
+    const long long T = bv.T, G = bv.G, B = bv.B, W32 = bv.W32, nC = bv.nC;
+    uint32_t *Hm = (uint32_t *)(base + bv.h), *tot = (uint32_t *)(base + bv.total);
+    uint32_t *start = (uint32_t *)(base + bv.start), *masks = (uint32_t *)(base + bv.mask);
+    uint4 *rect = (uint4 *)(base + bv.rect);
+    uint16_t *credit = bv.trunc ? (uint16_t *)(base + bv.credit) : nullptr;
+    uint32_t *bsat = bv.trunc ? (uint32_t *)(base + bv.sat) : nullptr;
+    int *P = bv.passes > 1 ? (int *)(base + bv.stopped) : nullptr;
+    if (bgs::bin_count_smem(bv.tiles_x, bv.tiles_y) > 48 * 1024)
+        BGS_CUDA(bgs::setup_bin_kernels(bv.tiles_x, bv.tiles_y), "bin smem attribute");
     // With truncation, in passes over the depth order ([0, B / 8), [B / 8, B / 2), [B / 2, B)):
     // a later pass leaves out the Gaussians all of whose tiles the earlier passes' credits
     // already certify as stopped (their entries lie past the ends of all their lists, so the
     // lists are the same)
     long long bounds[4] = {0, B, B, B};
-    int passes = 1;
-    if (bv.trunc && B >= 32) {
+    const int passes = bv.passes;
+    if (passes > 1) {
         bounds[1] = B / kBinPassDiv[0];
         bounds[2] = B / kBinPassDiv[1];
-        bounds[3] = B;
-        passes = 3;
-    }
-    uint32_t *masks = (uint32_t *)sl.mask.p;
-    int *P = nullptr;
-    if (passes > 1) {
-        BGS_TRY(ensure(p, sl.stopped, sizeof(int) * (size_t)(bv.tiles_x + 1) * (bv.tiles_y + 1), s, "bin_stopped"));
-        const size_t before = sl.stopped_sum.bytes;
-        BGS_TRY(ensure(p, sl.stopped_sum, sizeof(uint32_t) * T, s, "bin_stopped_sum"));
-        if (sl.stopped_sum.bytes != before)
-            BGS_CUDA(cudaMemsetAsync(sl.stopped_sum.p, 0, sl.stopped_sum.bytes, s), "clear bin_stopped_sum");
-        P = (int *)sl.stopped.p;
     }
     for (int k = 0; k < passes; ++k) {
         const int lo = (int)bounds[k], hi = (int)bounds[k + 1];
-        if (k > 0) BGS_CUDA(bgs::launch_bin_stopped(lo, bv.tiles_x, bv.tiles_y, credit, (uint32_t *)sl.stopped_sum.p, P, s), "bin_stopped");
+        if (k > 0) BGS_CUDA(bgs::launch_bin_stopped(lo, bv.tiles_x, bv.tiles_y, credit,
+                                                     (uint32_t *)p->bin_slot[slot].stopped_sum.p, P, s), "bin_stopped");
         BGS_CUDA(bgs::launch_bin_count(n, (int)G, lo, hi, order, means2D, radii, W, H, tw, th, Hm, rect, masks,
                                        (int)W32, k > 0 ? P : nullptr, s),
                  "bin_count");
@@ -774,14 +796,14 @@ int bin_view_a(bgs_plan *p, int slot, int v, long long n, const uint32_t *order,
         p->host_launches += k > 0 ? 4 : 1;
     }
     if (bv.trunc) p->host_launches += 1;
-    BGS_TRY(ensure(p, sl.items, sizeof(uint32_t) * (bv.nC + 1), s, "bin_items"));
     bgs::BinTiles &bt = bv.tiles;
     bt.T = (int)T, bt.tx = bv.tiles_x, bt.ty = bv.tiles_y, bt.B = (int)B, bt.nC = (int)nC, bt.v = v;
     bt.total = tot;
     bt.start = start;
     bt.ranges = reinterpret_cast<uint2 *>(ranges);
     bt.bsat = bsat;
-    bt.item_start = (uint32_t *)sl.items.p;
+    bt.item_start = (uint32_t *)(base + bv.items);
+    bt.warps = p->num_sms * bgs::kScatterBlocks;
     bt.only = only;
     bt.capacity = capacity;
     bt.host_k = capacity == kSyncCapacity ? p->host_k_dev : nullptr;  // a synchronous call reads it
@@ -793,16 +815,16 @@ int bin_view_a(bgs_plan *p, int slot, int v, long long n, const uint32_t *order,
 
 int bin_view_b(bgs_plan *p, int slot, int v, long long n, const BinView &bv, int W, int H, int tw, int th,
                uint32_t *point_list, long long capacity, cudaStream_t s) {
-    bgs_plan::BinSlot &sl = p->bin_slot[slot];
+    const char *base = (const char *)p->bin_slot[slot].arena.p;
     if (!bv.tiles.only) {
         BGS_CUDA(bgs::launch_bin_open(bv.tiles, s), "bin_open");
         p->host_launches += 1;
     }
-    BGS_CUDA(bgs::launch_bin_scatter(n, (int)bv.G, (int)bv.B, (int)bv.W32, (const uint4 *)sl.rect.p, W, H, tw, th,
-                                     (const uint32_t *)sl.h.p, (const uint32_t *)sl.start.p,
-                                     (const uint32_t *)sl.mask.p, point_list, capacity,
-                                     bv.trunc ? (const uint32_t *)sl.sat.p : nullptr, (const uint32_t *)sl.items.p,
-                                     p->num_sms, v, p->ctrl, s),
+    BGS_CUDA(bgs::launch_bin_scatter(n, (int)bv.G, (int)bv.B, (int)bv.W32, (const uint4 *)(base + bv.rect), W, H, tw,
+                                     th, (const uint32_t *)(base + bv.h), (const uint32_t *)(base + bv.start),
+                                     (const uint32_t *)(base + bv.mask), point_list, capacity,
+                                     bv.trunc ? (const uint32_t *)(base + bv.sat) : nullptr,
+                                     (const uint32_t *)(base + bv.items), p->num_sms, v, p->ctrl, s),
              "bin_scatter");
     p->host_launches += 1;
     return BGS_OK;
@@ -890,6 +912,8 @@ int bgs_bin_and_sort(bgs_plan *p, int64_t N, const float *means2D, const int32_t
     // (2) counting sort over tile rectangles
     if (counting) {
         BinView bv;
+        BGS_TRY(bin_sizes(p, N, conic_opacity != nullptr, W, H, tw, th, bv));
+        BGS_TRY(ensure_bin_slot(p, 0, bv.bytes, bv.passes > 1 ? bv.T : 0, s));
         // (the host checks K against the capacity)
         BGS_TRY(bin_view_a(p, 0, 0, N, order, means2D, radii, conic_opacity, W, H, tw, th, true, kSyncCapacity, ranges, bv, s));
         BGS_TRY(bin_view_b(p, 0, 0, N, bv, W, H, tw, th, point_list, capacity, s));
@@ -1350,6 +1374,17 @@ int bgs_bin_and_sort_batched(bgs_plan *p, int32_t V, const bgs_view *views, int6
         const int NS = std::min<int>(V, N < (2ll << 20) ? kSortStreams : kSortStreams / 2);
         auto stream_of = [&](int i) { return NS > 1 ? p->sort_stream[i] : s; };
         for (int i = 0; i < NS; ++i) BGS_TRY(ensure(p, p->sort_tmp[i], tmp, s, "sort_tmp"));
+        BinView bvs[bgs::kMaxViews];
+        for (int i = 0; i < NS; ++i) {  // a slot's scratch for the largest of its views, at once
+            size_t bytes = 0;
+            long long tiles = 0;
+            for (int v = i; v < V; v += NS) {
+                BGS_TRY(bin_sizes(p, N, conic_opacity != nullptr, Ws[v], Hs[v], tw, th, bvs[v]));
+                bytes = std::max(bytes, bvs[v].bytes);
+                if (bvs[v].passes > 1) tiles = std::max(tiles, bvs[v].T);
+            }
+            BGS_TRY(ensure_bin_slot(p, i, bytes, tiles, s));
+        }
         if (NS > 1) {
             BGS_CUDA(cudaEventRecord(p->sort_fork, s), "sort fork");
             for (int i = 0; i < NS; ++i)
@@ -1369,7 +1404,7 @@ int bgs_bin_and_sort_batched(bgs_plan *p, int32_t V, const bgs_view *views, int6
         for (int v = 0; v < V; ++v) {
             const int i = v % NS;
             cudaStream_t si = stream_of(i);
-            BinView bv;
+            BinView &bv = bvs[v];
             BGS_TRY(bin_view_a(p, i, v, N, order + (size_t)v * N, means2D, radii, conic_opacity, Ws[v], Hs[v], tw, th,
                                V == 1, sync ? kSyncCapacity : capacity, ranges + 2ull * vt.tile_base[v], bv, si));
             if (NS > 1) {
