@@ -200,6 +200,13 @@ int bgs_preprocess_backward(bgs_plan *plan, int64_t N, const float *means3D, con
                             const float *quats, const bgs_camera *cam, const int32_t *radii,
                             const float *dL_dmeans2D, const float *dL_dconic, const float *dL_ddepths,
                             float *dL_dmeans3D, float *dL_dlog_scales, float *dL_dquats, void *stream);
+/* The same from gradients of conic_opacity itself: dL_dconic_opacity [N,4] (16-byte aligned), whose
+   opacity column is copied to dL_dopacities [N] (of every Gaussian). */
+int bgs_preprocess_backward_rows(bgs_plan *plan, int64_t N, const float *means3D, const float *log_scales,
+                                 const float *quats, const bgs_camera *cam, const int32_t *radii,
+                                 const float *dL_dmeans2D, const float *dL_dconic_opacity, const float *dL_ddepths,
+                                 float *dL_dmeans3D, float *dL_dlog_scales, float *dL_dquats, float *dL_dopacities,
+                                 void *stream);
 
 /* ---- a2: binning: per-tile depth-ordered lists (point_list of Algorithms 1-6) --------
    Gaussian i with radius r > 0 covers the tiles x in [floor((u-r)/tw),
@@ -252,7 +259,8 @@ int bgs_render_forward(bgs_plan *plan, int64_t N, const float *means2D, const fl
    its final_T / n_contrib, dL_dcolor [3,H,W], dL_ddepth [H,W] (nullable),
    dL_dalpha [H,W] (nullable).  Outputs (overwritten): dL_dmeans2D [N,2],
    dL_dconic [N,3] (w.r.t. a, b, c exactly as used in power), dL_dopacity [N],
-   dL_dcolors [N,3], dL_ddepths [N] (nullable).  Where o exp(power) > 0.99 the alpha
+   dL_dcolors [N,3], dL_ddepths [N] (nullable).  With dL_dopacity = dL_dconic + 3 the two are
+   one array [N,4] (16-byte aligned) in the layout of conic_opacity.  Where o exp(power) > 0.99 the alpha
    clamp is active and the pair passes no gradient to o or to the Gaussian's shape.
    The arrays must hold what the forward read (final_T and n_contrib only describe that
    blend).  When they are the same arrays (pointers and sizes) as the plan's last forward,

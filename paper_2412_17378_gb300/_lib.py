@@ -34,8 +34,8 @@ EXPORTS = [
     "bgs_plan_num_sms", "bgs_last_error", "bgs_preprocess", "bgs_bin_and_sort", "bgs_render_forward",
     "bgs_render_backward", "bgs_probe_pipe_rates", "bgs_debug_exp2", "bgs_plan_timing", "bgs_plan_kernel_ms",
     "bgs_render_forward_noalloc", "bgs_preprocess_batched", "bgs_bin_and_sort_batched",
-    "bgs_preprocess_backward", "bgs_preprocess_backward_batched", "bgs_plan_selector", "bgs_plan_selector_reset",
-    "bgs_plan_inject_fault", "bgs_plan_selector_restore",
+    "bgs_preprocess_backward", "bgs_preprocess_backward_rows", "bgs_preprocess_backward_batched",
+    "bgs_plan_selector", "bgs_plan_selector_reset", "bgs_plan_inject_fault", "bgs_plan_selector_restore",
     "bgs_render_forward_batched", "bgs_render_backward_batched", "bgs_graph_begin", "bgs_graph_end",
     "bgs_graph_launch", "bgs_autotune_render", "bgs_render_forward_batched_vc", "bgs_render_backward_batched_vc",
     "bgs_sh_to_rgb", "bgs_sh_to_rgb_backward",
@@ -130,6 +130,7 @@ def load(build_if_needed: bool = True):
         VP = ctypes.POINTER(View)
         lib.bgs_preprocess_batched.argtypes = [P, i32, VP, i64, P, P, P, P, i32, i32, P, P, P, P, P, P]
         lib.bgs_preprocess_backward.argtypes = [P, i64, P, P, P, ctypes.POINTER(Camera), P, P, P, P, P, P, P, P]
+        lib.bgs_preprocess_backward_rows.argtypes = [P, i64, P, P, P, ctypes.POINTER(Camera), P, P, P, P, P, P, P, P, P]
         lib.bgs_preprocess_backward_batched.argtypes = [P, i32, VP, i64, P, P, P, P, P, P, P, P, P, P, P]
         lib.bgs_bin_and_sort_batched.argtypes = [P, i32, VP, i64, P, P, P, P, i32, i32, P, i64, P, i32,
                                                  ctypes.POINTER(i64), ctypes.POINTER(i64), P]

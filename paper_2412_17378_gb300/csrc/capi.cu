@@ -650,10 +650,15 @@ int bgs_preprocess(bgs_plan *p, int64_t N, const float *means3D, const float *lo
     return BGS_OK;
 }
 
-int bgs_preprocess_backward(bgs_plan *p, int64_t N, const float *means3D, const float *log_scales,
-                            const float *quats, const bgs_camera *cam, const int32_t *radii, const float *dL_dmeans2D,
+}  // extern "C"
+
+namespace {
+
+// dL_dopacities: dL_dconic holds (a, b, c, opacity) rows, whose fourth goes there
+int preprocess_backward_one(bgs_plan *p, int64_t N, const float *means3D, const float *log_scales, const float *quats,
+                            const bgs_camera *cam, const int32_t *radii, const float *dL_dmeans2D,
                             const float *dL_dconic, const float *dL_ddepths, float *dL_dmeans3D,
-                            float *dL_dlog_scales, float *dL_dquats, void *stream) {
+                            float *dL_dlog_scales, float *dL_dquats, float *dL_dopacities, cudaStream_t s) {
     if (!p || !cam) return fail(BGS_ERR_INVALID, "bgs_preprocess_backward: NULL plan or camera");
     if (N < 0 || N >= (1ll << 32)) return fail(BGS_ERR_INVALID, "bgs_preprocess_backward: N out of range");
     if (N > 0 && (!means3D || !log_scales || !quats || !radii || !dL_dmeans2D || !dL_dconic || !dL_dmeans3D ||
@@ -665,10 +670,35 @@ int bgs_preprocess_backward(bgs_plan *p, int64_t N, const float *means3D, const 
         return fail(BGS_ERR_INVALID, "bgs_preprocess_backward: focal lengths must be > 0");
     DeviceGuard g(p->device);
     BGS_CUDA(bgs::launch_preprocess_backward(N, 1, means3D, log_scales, quats, cam, radii, dL_dmeans2D, dL_dconic,
-                                             dL_ddepths, dL_dmeans3D, dL_dlog_scales, dL_dquats, (cudaStream_t)stream),
+                                             dL_ddepths, dL_dmeans3D, dL_dlog_scales, dL_dquats, dL_dopacities, s),
              "preprocess_backward");
     if (N > 0) p->host_launches += 1;
     return BGS_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int bgs_preprocess_backward(bgs_plan *p, int64_t N, const float *means3D, const float *log_scales,
+                            const float *quats, const bgs_camera *cam, const int32_t *radii, const float *dL_dmeans2D,
+                            const float *dL_dconic, const float *dL_ddepths, float *dL_dmeans3D,
+                            float *dL_dlog_scales, float *dL_dquats, void *stream) {
+    return preprocess_backward_one(p, N, means3D, log_scales, quats, cam, radii, dL_dmeans2D, dL_dconic, dL_ddepths,
+                                   dL_dmeans3D, dL_dlog_scales, dL_dquats, nullptr, (cudaStream_t)stream);
+}
+
+int bgs_preprocess_backward_rows(bgs_plan *p, int64_t N, const float *means3D, const float *log_scales,
+                                 const float *quats, const bgs_camera *cam, const int32_t *radii,
+                                 const float *dL_dmeans2D, const float *dL_dconic_opacity, const float *dL_ddepths,
+                                 float *dL_dmeans3D, float *dL_dlog_scales, float *dL_dquats, float *dL_dopacities,
+                                 void *stream) {
+    if (N > 0 && !dL_dopacities) return fail(BGS_ERR_INVALID, "bgs_preprocess_backward_rows: NULL array");
+    if (((uintptr_t)dL_dconic_opacity) & 15)
+        return fail(BGS_ERR_INVALID, "bgs_preprocess_backward_rows: dL_dconic_opacity alignment");
+    return preprocess_backward_one(p, N, means3D, log_scales, quats, cam, radii, dL_dmeans2D, dL_dconic_opacity,
+                                   dL_ddepths, dL_dmeans3D, dL_dlog_scales, dL_dquats, dL_dopacities,
+                                   (cudaStream_t)stream);
 }
 
 }  // extern "C"
@@ -1081,6 +1111,8 @@ int render_backward_impl(bgs_plan *p, const bgs::ViewTable &vt, const bgs::ViewG
                          int tw, int th, const float *bg, int mode, float *dL_dmeans2D, float *dL_dconic,
                          float *dL_dopacity, float *dL_dcolors, float *dL_ddepths, cudaStream_t s) {
     if (n_records == 0) return BGS_OK;
+    if (n_records > 1 && dL_dopacity == dL_dconic + 3 && (((uintptr_t)dL_dconic) & 15))
+        return fail(BGS_ERR_INVALID, "interleaved conic and opacity gradients want a 16-byte aligned array");
     BGS_TRY(ensure(p, p->grad_acc, sizeof(bgs::Rec) * n_records, s, "grad_acc"));
     BGS_CUDA(cudaMemsetAsync(p->grad_acc.p, 0, sizeof(bgs::Rec) * n_records, s), "clear grad_acc");
     bgs::BwdArgs a;
@@ -1311,7 +1343,8 @@ int bgs_preprocess_backward_batched(bgs_plan *p, int32_t V, const bgs_view *view
     }
     DeviceGuard g(p->device);
     BGS_CUDA(bgs::launch_preprocess_backward(N, V, means3D, log_scales, quats, cams, radii, dL_dmeans2D, dL_dconic,
-                                             dL_ddepths, dL_dmeans3D, dL_dlog_scales, dL_dquats, (cudaStream_t)stream),
+                                             dL_ddepths, dL_dmeans3D, dL_dlog_scales, dL_dquats, nullptr,
+                                             (cudaStream_t)stream),
              "preprocess_backward_batched");
     if (N > 0) p->host_launches += 1;
     return BGS_OK;

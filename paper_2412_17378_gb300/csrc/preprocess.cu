@@ -204,6 +204,9 @@ __global__ void __launch_bounds__(128) k_preprocess(long long N, const float *__
 //   means2D = (fx x / z + cx, fy y / z + cy), depth = z, t = W p + w;
 //   Sigma = M M^T, M = R S: dL/dM = 2 dL/dSigma M, dL/dlog s_k = s_k sum_r dL/dM_rk R_rk,
 //   dL/dR = dL/dM S, then R(q) and the Jacobian of q / |q|.
+// Rows: the conic gradients are the first three of rows of four floats, whose fourth, the opacity's
+// gradient, goes to dL_dopacities as it is.
+template <bool Rows>
 __global__ void __launch_bounds__(128, 5) k_preprocess_backward(long long N, const float *__restrict__ means3D,
                                                              const float *__restrict__ log_scales,
                                                              const float *__restrict__ quats, const CamTable ct,
@@ -213,7 +216,8 @@ __global__ void __launch_bounds__(128, 5) k_preprocess_backward(long long N, con
                                                              const float *__restrict__ dL_ddepths,
                                                              float *__restrict__ dL_dmeans3D,
                                                              float *__restrict__ dL_dlog_scales,
-                                                             float *__restrict__ dL_dquats) {
+                                                             float *__restrict__ dL_dquats,
+                                                             float *__restrict__ dL_dopacities) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= N) return;
     // summed over the views; gls and gR (dL/dR) still without their factors 2 s_k^2, which like
@@ -228,14 +232,19 @@ __global__ void __launch_bounds__(128, 5) k_preprocess_backward(long long N, con
     struct In {
         int r;
         float2 m;
-        float a, b, c, d;
+        float a, b, c, d, o;
     } next;
     uint32_t rec = (uint32_t)g;  // V N < 2^32
     auto load = [&](uint32_t k) {
         In i;
         i.r = radii[k];
         i.m = dL_dmeans2D[k];
-        i.a = dL_dconic[3ull * k], i.b = dL_dconic[3ull * k + 1], i.c = dL_dconic[3ull * k + 2];
+        if (Rows) {
+            const float4 c = reinterpret_cast<const float4 *>(dL_dconic)[k];
+            i.a = c.x, i.b = c.y, i.c = c.z, i.o = c.w;
+        } else {
+            i.a = dL_dconic[3ull * k], i.b = dL_dconic[3ull * k + 1], i.c = dL_dconic[3ull * k + 2];
+        }
         i.d = dL_ddepths ? dL_ddepths[k] : 0.f;
         return i;
     };
@@ -244,6 +253,7 @@ __global__ void __launch_bounds__(128, 5) k_preprocess_backward(long long N, con
         const In in = next;
         rec += (uint32_t)N;
         if (view + 1 < ct.V) next = load(rec);
+        if (Rows) dL_dopacities[rec - (uint32_t)N] = in.o;
         if (in.r <= 0) continue;
         const CamDev &cam = ct.cam[view];
         Proj o = frame;
@@ -382,15 +392,17 @@ cudaError_t launch_preprocess(long long N, int V, const float *means3D, const fl
 cudaError_t launch_preprocess_backward(long long N, int V, const float *means3D, const float *log_scales,
                                        const float *quats, const bgs_camera *cams, const int *radii,
                                        const float *dL_dmeans2D, const float *dL_dconic, const float *dL_ddepths,
-                                       float *dL_dmeans3D, float *dL_dlog_scales, float *dL_dquats, cudaStream_t s) {
+                                       float *dL_dmeans3D, float *dL_dlog_scales, float *dL_dquats,
+                                       float *dL_dopacities, cudaStream_t s) {
     if (V < 1 || V > kMaxViews) return cudaErrorInvalidValue;
     CamTable ct;
     ct.V = V;
     for (int v = 0; v < V; ++v) ct.cam[v] = cam_dev(cams[v], 16, 16);
     if (N == 0) return cudaSuccess;
-    k_preprocess_backward<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(
+    auto *kernel = dL_dopacities ? k_preprocess_backward<true> : k_preprocess_backward<false>;
+    kernel<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(
         N, means3D, log_scales, quats, ct, radii, reinterpret_cast<const float2 *>(dL_dmeans2D), dL_dconic,
-        dL_ddepths, dL_dmeans3D, dL_dlog_scales, dL_dquats);
+        dL_ddepths, dL_dmeans3D, dL_dlog_scales, dL_dquats, dL_dopacities);
     return cudaGetLastError();
 }
 

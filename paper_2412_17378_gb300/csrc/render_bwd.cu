@@ -599,7 +599,7 @@ __device__ __forceinline__ void finalize_record(long long i, const float4 *__res
                                                 const float4 *__restrict__ conic_opacity,
                                                 float *__restrict__ dL_dmeans2D, float *__restrict__ dL_dconic,
                                                 float *__restrict__ dL_dopacity, float *__restrict__ dL_ddepths,
-                                                float &cr, float &cg, float &cb) {
+                                                bool rows, float &cr, float &cg, float &cb) {
     const float4 a0 = acc[3 * i], a1 = acc[3 * i + 1], a2 = acc[3 * i + 2];
     const float4 co = conic_opacity[i];
     // power = ln2 * power2 with power2 = qa dx^2 + qb dx dy + qc dy^2 and (qa, qb, qc) the
@@ -609,11 +609,16 @@ __device__ __forceinline__ void finalize_record(long long i, const float4 *__res
     const float qa = -0.5f * kLog2e * co.x, qb = -kLog2e * co.y, qc = -0.5f * kLog2e * co.z;
     dL_dmeans2D[2 * i] = kLn2 * (2.f * qa * a0.x + qb * a0.y);
     dL_dmeans2D[2 * i + 1] = kLn2 * (2.f * qc * a0.y + qb * a0.x);
-    dL_dconic[3 * i] = -0.5f * a0.z;
-    dL_dconic[3 * i + 1] = -a0.w;
-    dL_dconic[3 * i + 2] = -0.5f * a1.x;
     // sum gp / o = sum G dL/dalpha (a record with o = 0 has alpha = 0 everywhere: no pair)
-    dL_dopacity[i] = co.w > 0.f ? a1.y / co.w : 0.f;
+    const float go = co.w > 0.f ? a1.y / co.w : 0.f;
+    if (rows) {
+        reinterpret_cast<float4 *>(dL_dconic)[i] = make_float4(-0.5f * a0.z, -a0.w, -0.5f * a1.x, go);
+    } else {
+        dL_dconic[3 * i] = -0.5f * a0.z;
+        dL_dconic[3 * i + 1] = -a0.w;
+        dL_dconic[3 * i + 2] = -0.5f * a1.x;
+        dL_dopacity[i] = go;
+    }
     if (dL_ddepths) dL_ddepths[i] = a2.y;
     cr += a1.z;
     cg += a1.w;
@@ -624,7 +629,7 @@ __global__ void __launch_bounds__(256) k_grad_finalize(long long N, long long n_
                                                        const float4 *__restrict__ conic_opacity,
                                                        float *__restrict__ dL_dmeans2D, float *__restrict__ dL_dconic,
                                                        float *__restrict__ dL_dopacity, float *__restrict__ dL_dcolors,
-                                                       float *__restrict__ dL_ddepths,
+                                                       float *__restrict__ dL_ddepths, bool rows,
                                                        const unsigned int *__restrict__ warp_items, int n_warps,
                                                        DevCtrl *ctrl) {
     if (blockIdx.x == 0 && n_warps > 0) {
@@ -648,7 +653,7 @@ __global__ void __launch_bounds__(256) k_grad_finalize(long long N, long long n_
     if (g >= stride) return;
     float cr = 0.f, cg = 0.f, cb = 0.f;
     for (long long i = g; i < N; i += stride)
-        finalize_record(i, acc, conic_opacity, dL_dmeans2D, dL_dconic, dL_dopacity, dL_ddepths, cr, cg, cb);
+        finalize_record(i, acc, conic_opacity, dL_dmeans2D, dL_dconic, dL_dopacity, dL_ddepths, rows, cr, cg, cb);
     if (n_colors > 0) {
         dL_dcolors[3 * g] = cr;
         dL_dcolors[3 * g + 1] = cg;
@@ -662,9 +667,12 @@ cudaError_t launch_grad_finalize(long long N, long long n_colors, const float4 *
                                  cudaStream_t s) {
     if (N == 0 && n_warps == 0) return cudaSuccess;
     const long long threads = (n_colors > 0 && n_colors < N) ? n_colors : N;
+    // an opacity gradient right behind the first conic gradient: the two interleaved, rows of four
+    // floats, the layout of conic_opacity, so that no pass has to bring them together (29 us for 3M)
+    const bool rows = N > 1 && dL_dopacity == dL_dconic + 3;
     k_grad_finalize<<<(unsigned)std::max<long long>(1, (threads + 255) / 256), 256, 0, s>>>(
         N, n_colors, acc, reinterpret_cast<const float4 *>(conic_opacity), dL_dmeans2D, dL_dconic, dL_dopacity,
-        dL_dcolors, dL_ddepths, warp_items, n_warps, ctrl);
+        dL_dcolors, dL_ddepths, rows, warp_items, n_warps, ctrl);
     return cudaGetLastError();
 }
 

@@ -10,6 +10,7 @@ bgs_render_backward.
 from __future__ import annotations
 
 import ctypes
+import functools
 
 import numpy as np
 import torch
@@ -285,7 +286,8 @@ def render_forward(plan: Plan, means2D, conic_opacity, colors, depths, point_lis
 def render_backward(plan: Plan, means2D, conic_opacity, colors, depths, point_list, num_entries: int, ranges,
                     W: int, H: int, final_T, n_contrib, dL_dcolor, dL_ddepth=None, dL_dalpha=None, tile=(16, 16),
                     bg=(0.0, 0.0, 0.0), mode="auto", out=None):
-    """bgs_render_backward: returns dict(means2D [N,2], conic [N,3], opacity [N], colors [N,3], depths [N])."""
+    """bgs_render_backward: returns dict(means2D [N,2], conic [N,3], opacity [N], colors [N,3], depths [N]).
+    ``out`` may hold conic_opacity [N,4] in place of conic and opacity."""
     N = means2D.shape[0]
     _req(final_T, "final_T", torch.float32, (H, W))
     _req(n_contrib, "n_contrib", torch.int32, (H, W))
@@ -299,13 +301,17 @@ def render_backward(plan: Plan, means2D, conic_opacity, colors, depths, point_li
         out = dict(means2D=torch.empty((N, 2), device=dev), conic=torch.empty((N, 3), device=dev),
                    opacity=torch.empty(N, device=dev), colors=torch.empty((N, 3), device=dev),
                    depths=torch.empty(N, device=dev))
+    conic, opacity = _ptr(out.get("conic")), _ptr(out.get("opacity"))
+    if "conic_opacity" in out:  # interleaved
+        rows = out["conic_opacity"]
+        conic, opacity = _ptr(rows), ctypes.c_void_p(rows.data_ptr() + 12) if N > 0 else None
     bgv = (ctypes.c_float * 3)(*[float(v) for v in bg])
     m = MODES[mode] if isinstance(mode, str) else int(mode)
     check(plan._lib.bgs_render_backward(plan.handle, N, _ptr(means2D), _ptr(conic_opacity), _ptr(colors),
                                         _ptr(depths), _ptr(point_list), int(num_entries), _ptr(ranges), W, H,
                                         tile[0], tile[1], bgv, m, _ptr(final_T), _ptr(n_contrib), _ptr(dL_dcolor),
-                                        _ptr(dL_ddepth), _ptr(dL_dalpha), _ptr(out["means2D"]), _ptr(out["conic"]),
-                                        _ptr(out["opacity"]), _ptr(out["colors"]), _ptr(out.get("depths")),
+                                        _ptr(dL_ddepth), _ptr(dL_dalpha), _ptr(out["means2D"]), conic, opacity,
+                                        _ptr(out["colors"]), _ptr(out.get("depths")),
                                         _stream(dev)), "bgs_render_backward")
     return out
 
@@ -359,19 +365,21 @@ class RenderFunction(torch.autograd.Function):
     @staticmethod
     def backward(ctx, g_color, g_depth, g_alpha, _g_T, _g_n):
         means2D, conic_opacity, colors, depths, point_list, ranges, final_T, n_contrib = ctx.saved_tensors
+        # (gradients of conic_opacity as one array: no pass joins or splits them)
+        N, new = means2D.shape[0], functools.partial(torch.empty, device=means2D.device)
+        out = dict(means2D=new((N, 2)), conic_opacity=new((N, 4)), colors=new((N, 3)), depths=new(N))
         g = render_backward(ctx.plan, means2D, conic_opacity, colors, depths, point_list, ctx.K, ranges, ctx.W,
                             ctx.H, final_T, n_contrib,
                             g_color.contiguous() if g_color is not None else torch.zeros_like(final_T).expand(3, -1, -1).contiguous(),
                             None if g_depth is None else g_depth.contiguous(),
                             None if g_alpha is None else g_alpha.contiguous(),
-                            ctx.tile, ctx.bg, ctx.mode)
-        d_conic = torch.cat([g["conic"], g["opacity"][:, None]], 1)
-        return g["means2D"], d_conic, g["colors"], g["depths"], None, None, None, None, None, None, None
+                            ctx.tile, ctx.bg, ctx.mode, out)
+        return g["means2D"], g["conic_opacity"], g["colors"], g["depths"], None, None, None, None, None, None, None
 
 
 class PreprocessFunction(torch.autograd.Function):
     """Differentiable projection (Eq. 1-3): (means3D, log_scales, quats, opacities) ->
-    (means2D, conic_opacity, depths, radii).  The backward calls bgs_preprocess_backward;
+    (means2D, conic_opacity, depths, radii).  The backward calls bgs_preprocess_backward_rows;
     the opacity column of conic_opacity passes its gradient straight to opacities."""
 
     @staticmethod
@@ -390,10 +398,21 @@ class PreprocessFunction(torch.autograd.Function):
         N = m3.shape[0]
         z = lambda *shape: torch.zeros(shape, device=m3.device)
         gm = g_means2D.contiguous() if g_means2D is not None else z(N, 2)
-        gco = g_conic_opacity if g_conic_opacity is not None else z(N, 4)
+        gco = g_conic_opacity.contiguous() if g_conic_opacity is not None else z(N, 4)
         gd = g_depths.contiguous() if g_depths is not None else None
-        g = preprocess_backward(ctx.plan, m3, ls, q, ctx.cam, radii, gm, gco[:, :3].contiguous(), gd)
-        return g["means3D"], g["log_scales"], g["quats"], gco[:, 3].contiguous(), None, None, None
+        if gco.data_ptr() & 15:
+            gco = gco.clone()
+        _req(gm, "dL_dmeans2D", torch.float32, (N, 2))
+        _req(gco, "dL_dconic_opacity", torch.float32, (N, 4))
+        if gd is not None:
+            _req(gd, "dL_ddepths", torch.float32, (N,))
+        g, d_opacities = _grads_out(N, m3.device, None), torch.empty(N, device=m3.device)
+        c = camera_struct(ctx.cam)
+        check(ctx.plan._lib.bgs_preprocess_backward_rows(
+            ctx.plan.handle, N, _ptr(m3), _ptr(ls), _ptr(q), ctypes.byref(c), _ptr(radii), _ptr(gm), _ptr(gco),
+            _ptr(gd), _ptr(g["means3D"]), _ptr(g["log_scales"]), _ptr(g["quats"]), _ptr(d_opacities),
+            _stream(m3.device)), "bgs_preprocess_backward_rows")
+        return g["means3D"], g["log_scales"], g["quats"], d_opacities, None, None, None
 
 
 def render(plan: Plan, means2D, conic_opacity, colors, depths, binning, W, H, tile=(16, 16), bg=(0.0, 0.0, 0.0),
