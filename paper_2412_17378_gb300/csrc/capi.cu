@@ -94,6 +94,11 @@ struct bgs_plan {
     unsigned long long *host_k = nullptr, *host_k_dev = nullptr;  // mapped: the last call's entry count
     // render
     Buf recs, tile_idx, items, grad_acc, warp_items;  // tile_idx: each tile's slot in its work-list bucket
+    // Leading bytes of grad_acc that are zero between calls: a backward's last kernel, which reads
+    // every accumulator, clears those that hold something (a pass that cleared them all first
+    // wrote 48 bytes a record, most of them never touched: nine views of 4M Gaussians
+    // 12.01 -> 11.79 ms, a 3M training step 1740 -> 1717 us)
+    size_t grad_clear = 0;
     Buf gw_exoff, gw_ent, gw_tile, gw_done, gw_sum;  // Gaussian-wise segments: per-tile later-segment
                                                      // offsets, entries, per-tile entry numbers, per-block
                                                      // flags, per-pixel summaries
@@ -154,6 +159,7 @@ int ensure(bgs_plan *p, Buf &b, size_t bytes, cudaStream_t s, const char *what) 
     if (&b == &p->recs) p->rec_valid = false;
     if (&b == &p->items) p->wl_valid = false;
     if (&b == &p->gidx) p->iota_n = 0;
+    if (&b == &p->grad_acc) p->grad_clear = 0;
     if (b.p) {
         cudaError_t e = cudaFree(b.p);
         b.p = nullptr;
@@ -1114,7 +1120,12 @@ int render_backward_impl(bgs_plan *p, const bgs::ViewTable &vt, const bgs::ViewG
     if (n_records > 1 && dL_dopacity == dL_dconic + 3 && (((uintptr_t)dL_dconic) & 15))
         return fail(BGS_ERR_INVALID, "interleaved conic and opacity gradients want a 16-byte aligned array");
     BGS_TRY(ensure(p, p->grad_acc, sizeof(bgs::Rec) * n_records, s, "grad_acc"));
-    BGS_CUDA(cudaMemsetAsync(p->grad_acc.p, 0, sizeof(bgs::Rec) * n_records, s), "clear grad_acc");
+    const size_t acc_bytes = sizeof(bgs::Rec) * n_records, clear = p->grad_clear;
+    if (clear < acc_bytes)
+        BGS_CUDA(cudaMemsetAsync(p->grad_acc.p, 0, acc_bytes, s), "clear grad_acc");
+    // (not clear until the last kernel is launched; a captured call runs later, if at all)
+    const bool later = capturing(s);
+    if (!later) p->grad_clear = 0;
     bgs::BwdArgs a;
     memset(&a, 0, sizeof a);
     a.bseg_mode = -1;
@@ -1191,11 +1202,12 @@ int render_backward_impl(bgs_plan *p, const bgs::ViewTable &vt, const bgs::ViewG
         kt.stop();
         p->host_launches += 1;  // kernel
     }
-    BGS_CUDA(bgs::launch_grad_finalize(n_records, n_colors, (const float4 *)p->grad_acc.p, conic_opacity, dL_dmeans2D,
+    BGS_CUDA(bgs::launch_grad_finalize(n_records, n_colors, (float4 *)p->grad_acc.p, conic_opacity, dL_dmeans2D,
                                        dL_dconic, dL_dopacity, dL_dcolors, dL_ddepths,
                                        (const unsigned int *)p->warp_items.p, n_warps, p->ctrl, s),
              "grad_finalize");
     p->host_launches += 1;  // finalize
+    if (!later) p->grad_clear = std::max(clear, acc_bytes);
     return BGS_OK;
 }
 

@@ -595,12 +595,18 @@ cudaError_t launch_backward_balanced(const BwdArgs &a, int grid, cudaStream_t s)
 // batched call when n_colors < N (records g, g + n_colors, ... are Gaussian g seen from
 // each view): then a thread takes Gaussian g, finalizes its records one view after another
 // and writes its colour gradient summed over them, reading each accumulator row once.
-__device__ __forceinline__ void finalize_record(long long i, const float4 *__restrict__ acc,
+__device__ __forceinline__ void finalize_record(long long i, float4 *__restrict__ acc,
                                                 const float4 *__restrict__ conic_opacity,
                                                 float *__restrict__ dL_dmeans2D, float *__restrict__ dL_dconic,
                                                 float *__restrict__ dL_dopacity, float *__restrict__ dL_ddepths,
                                                 bool rows, float &cr, float &cg, float &cb) {
     const float4 a0 = acc[3 * i], a1 = acc[3 * i + 1], a2 = acc[3 * i + 2];
+    auto bits = [](float4 x) {
+        return __float_as_uint(x.x) | __float_as_uint(x.y) | __float_as_uint(x.z) | __float_as_uint(x.w);
+    };
+    if ((bits(a0) | bits(a1) | bits(a2)) != 0u) {  // leave the accumulators clear
+        acc[3 * i] = acc[3 * i + 1] = acc[3 * i + 2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     const float4 co = conic_opacity[i];
     // power = ln2 * power2 with power2 = qa dx^2 + qb dx dy + qc dy^2 and (qa, qb, qc) the
     // record's pre-scaled conic; d power / d mean = ln2 (2 qa dx + qb dy, 2 qc dy + qb dx),
@@ -625,7 +631,7 @@ __device__ __forceinline__ void finalize_record(long long i, const float4 *__res
     cb += a2.x;
 }
 
-__global__ void __launch_bounds__(256) k_grad_finalize(long long N, long long n_colors, const float4 *__restrict__ acc,
+__global__ void __launch_bounds__(256) k_grad_finalize(long long N, long long n_colors, float4 *__restrict__ acc,
                                                        const float4 *__restrict__ conic_opacity,
                                                        float *__restrict__ dL_dmeans2D, float *__restrict__ dL_dconic,
                                                        float *__restrict__ dL_dopacity, float *__restrict__ dL_dcolors,
@@ -661,7 +667,7 @@ __global__ void __launch_bounds__(256) k_grad_finalize(long long N, long long n_
     }
 }
 
-cudaError_t launch_grad_finalize(long long N, long long n_colors, const float4 *acc, const float *conic_opacity,
+cudaError_t launch_grad_finalize(long long N, long long n_colors, float4 *acc, const float *conic_opacity,
                                  float *dL_dmeans2D, float *dL_dconic, float *dL_dopacity, float *dL_dcolors,
                                  float *dL_ddepths, const unsigned int *warp_items, int n_warps, DevCtrl *ctrl,
                                  cudaStream_t s) {
