@@ -178,9 +178,9 @@ struct __align__(16) Hit {
 
 // Gathers the warp's next 32 records (lane's index g, valid: within the list, position pos),
 // tests each against the pixel block and packs those that reach it into buf in list order.
-// Returns their number.
+// Returns their number; *odd: one of them is (record_odd).
 __device__ __forceinline__ int stage_window(const FwdArgs &a, uint32_t g, bool valid, uint32_t pos, float bcx,
-                                            float bcy, float hw, float hh, Hit *buf, int lane) {
+                                            float bcy, float hw, float hh, Hit *buf, int lane, bool *odd = nullptr) {
     bool hit = false;
     Rec r;
     if (valid) {
@@ -192,6 +192,7 @@ __device__ __forceinline__ int stage_window(const FwdArgs &a, uint32_t g, bool v
         }
     }
     const unsigned live = __ballot_sync(kFull, hit);
+    if (odd) *odd = __any_sync(kFull, hit && r.b.w != 0.f);
     if (hit) {
         Hit *h = buf + __popc(live & ((1u << lane) - 1u));
         *reinterpret_cast<float4 *>(h) = make_float4(r.a.x, r.a.z, r.a.w, __uint_as_float(pos));
@@ -210,16 +211,45 @@ struct PixAcc {
     static constexpr int NP = (Q + 1) / 2;
     F2 npy[NP];  // -y; -infinity once a pixel has stopped (and outside the image): no pair passes
     F2 T[NP], c0[NP], c1[NP], c2[NP], D[NP];
-    int last[2 * NP], neval[2 * NP], nacc;
+    int last[2 * NP], nacc;
+    int *neval;  // the lane's slots in shared memory, 32 apart: written where a pixel stops, read at the end
 };
+
+// Where a pixel's t = T (1 - alpha) falls below the stop threshold: the pair is not accumulated.
+template <int Q, bool Near>
+__device__ __forceinline__ void stop_pixels(F2 *nal, F2 *tt, const F2 *T, bool *v, int pos, int nacc, PixAcc<Q> &s,
+                                            bool *near) {
+#pragma unroll
+    for (int p = 0; p < PixAcc<Q>::NP; ++p) {
+        float2 a = f2_split(nal[p]), t = f2_split(tt[p]), y = f2_split(s.npy[p]);
+        const float2 T0 = f2_split(T[p]);
+        if (Near) {
+            const float m = kTMin * 6e-8f * (3.f * (float)nacc + 16.f);
+            *near = *near || nacc > 1000 || fabsf(t.x - kTMin) <= m || fabsf(t.y - kTMin) <= m;
+        }
+        if (t.x < kTMin) {
+            a.x = 0.f, t.x = T0.x, y.x = -INFINITY;
+            v[2 * p] = false;
+            s.neval[32 * (2 * p)] = pos;
+        }
+        if (t.y < kTMin) {
+            a.y = 0.f, t.y = T0.y, y.y = -INFINITY;
+            v[2 * p + 1] = false;
+            s.neval[32 * (2 * p + 1)] = pos;
+        }
+        nal[p] = f2(a.x, a.y);
+        tt[p] = f2(t.x, t.y);
+        s.npy[p] = f2(y.x, y.y);
+    }
+}
 
 // One record on the lane's pixels: the rule of the scalar kernels, bit for bit, two pixels per
 // instruction.  A pair that is not accumulated has alpha = 0, which leaves T and the sums as
 // they are, so nothing branches but a pixel's stop.  Odd = false (record_odd): the pair rule
 // without its sign test and clamp; Odd = true: in full, a masked pair's colour left out by
 // selection.  Against a branch per pair in scalar code the kernel issues 15-23 % fewer
-// instructions (the ALU pipe, at 50-54 %, is then its busiest) and takes 2.04 instead of 2.12
-// ms on the 9-view 4M-Gaussian step, 173-189 instead of 207 us on a 720p early-stage view.
+// instructions and takes 2.04 instead of 2.12 ms on the 9-view 4M-Gaussian step, 173-189 instead
+// of 207 us on a 720p early-stage view.
 template <int Q, bool Odd, bool Near = false>
 __device__ __forceinline__ void blend_hit(const Hit &h, float pxf, PixAcc<Q> &s, bool *near = nullptr) {
     constexpr int NP = PixAcc<Q>::NP;
@@ -247,28 +277,7 @@ __device__ __forceinline__ void blend_hit(const Hit &h, float pxf, PixAcc<Q> &s,
         tmin = fminf(tmin, fminf(t.x, t.y));
     }
     if (tmin < (Near ? 1.0002f * kTMin : kTMin)) {  // a pixel stops here: the pair is not accumulated
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            float2 a = f2_split(nal[p]), t = f2_split(tt[p]), y = f2_split(s.npy[p]);
-            const float2 T = f2_split(s.T[p]);
-            if (Near) {
-                const float m = kTMin * 6e-8f * (3.f * (float)s.nacc + 16.f);
-                *near = *near || s.nacc > 1000 || fabsf(t.x - kTMin) <= m || fabsf(t.y - kTMin) <= m;
-            }
-            if (t.x < kTMin) {
-                a.x = 0.f, t.x = T.x, y.x = -INFINITY;
-                v[2 * p] = false;
-                s.neval[2 * p] = pos;
-            }
-            if (t.y < kTMin) {
-                a.y = 0.f, t.y = T.y, y.y = -INFINITY;
-                v[2 * p + 1] = false;
-                s.neval[2 * p + 1] = pos;
-            }
-            nal[p] = f2(a.x, a.y);
-            tt[p] = f2(t.x, t.y);
-            s.npy[p] = f2(y.x, y.y);
-        }
+        stop_pixels<Q, Near>(nal, tt, s.T, v, pos, s.nacc, s, near);
     }
     const ulonglong2 h3 = *reinterpret_cast<const ulonglong2 *>(&h.g);
     const F2 h4 = h.d;
@@ -293,6 +302,80 @@ __device__ __forceinline__ void blend_hit(const Hit &h, float pxf, PixAcc<Q> &s,
     }
 }
 
+// The lane's pixels' -alpha T factors of one plain record (record_odd = 0), as blend_hit takes them.
+template <int Q>
+__device__ __forceinline__ void plain_alpha(const Hit &h, float pxf, const PixAcc<Q> &s, F2 *nal, bool *v) {
+    const float4 h0 = *reinterpret_cast<const float4 *>(&h);
+    const ulonglong2 h1 = *reinterpret_cast<const ulonglong2 *>(&h.my);
+    const F2 o = h.o;
+    const float dx = __fsub_rn(h0.x, pxf), hx = __fmul_rn(__fmul_rn(h0.y, dx), dx), bx = __fmul_rn(h0.z, dx);
+    const F2 hx2 = f2(hx, hx), bx2 = f2(bx, bx);
+#pragma unroll
+    for (int p = 0; p < PixAcc<Q>::NP; ++p) {
+        const F2 dy = f2_add(h1.x, s.npy[p]);
+        const float2 e = f2_split(f2_fma(dy, f2_fma(h1.y, dy, bx2), hx2));
+        const float2 oG = f2_split(f2_mul(o, f2(ex2_approx(e.x), Q == 1 ? 0.f : ex2_approx(e.y))));
+        v[2 * p] = oG.x >= kAlphaMin;
+        v[2 * p + 1] = Q > 1 && oG.y >= kAlphaMin;
+        nal[p] = f2(v[2 * p] ? -oG.x : 0.f, v[2 * p + 1] ? -oG.y : 0.f);
+    }
+}
+
+// Two plain records after one another on the lane's pixels: the arithmetic of blend_hit on each. A
+// pixel's alphas do not depend on its transmittance, which alone runs through both, so one
+// record's exponentials cover the other's latency (24 warps an SM left 27 % of the issue slots
+// empty), and the stop is tested once for both.  A stop is resolved in place, by the lane that
+// has it: sent back to blend_hit, the lanes of a warp drift apart by a record (the 9-view step
+// 11.84 instead of 11.78 ms), and sent back together they lose the second record's work (11.94).
+// Against one record at a time a 600k-Gaussian 1080p frame takes 533 instead of 541 us, a 720p
+// early-stage render and backward 545 instead of 559, a 1080p one under the plan's defaults 826
+// instead of 867.
+template <int Q, bool Near>
+__device__ __forceinline__ void blend_two(const Hit &ha, const Hit &hb, float pxf, PixAcc<Q> &s, bool *near) {
+    constexpr int NP = PixAcc<Q>::NP;
+    F2 na[NP], nb[NP], ta[NP], tb[NP];
+    bool va[2 * NP], vb[2 * NP];
+    plain_alpha<Q>(ha, pxf, s, na, va);
+    plain_alpha<Q>(hb, pxf, s, nb, vb);
+    float tmin = 1.f;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        ta[p] = f2_fma(s.T[p], na[p], s.T[p]);  // next_T
+        tb[p] = f2_fma(ta[p], nb[p], ta[p]);    // (at most ta)
+        const float2 t = f2_split(tb[p]);
+        tmin = fminf(tmin, fminf(t.x, t.y));
+    }
+    const int pa = (int)ha.pos, pb = (int)hb.pos;
+    if (tmin < (Near ? 1.0002f * kTMin : kTMin)) {  // a pixel stops, at the first (and meets no second) or the second
+        stop_pixels<Q, Near>(na, ta, s.T, va, pa, s.nacc, s, near);
+        int nacc = s.nacc;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const float2 y = f2_split(s.npy[p]), b = f2_split(nb[p]);
+            vb[2 * p] = vb[2 * p] && y.x != -INFINITY;
+            vb[2 * p + 1] = vb[2 * p + 1] && y.y != -INFINITY;
+            nb[p] = f2(vb[2 * p] ? b.x : 0.f, vb[2 * p + 1] ? b.y : 0.f);
+            tb[p] = f2_fma(ta[p], nb[p], ta[p]);
+            nacc += (va[2 * p] ? 1 : 0) + (va[2 * p + 1] ? 1 : 0);
+        }
+        stop_pixels<Q, Near>(nb, tb, ta, vb, pb, nacc, s, near);
+    }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        const F2 wa = f2_mul(na[p], s.T[p]), wb = f2_mul(nb[p], ta[p]);
+        s.c0[p] = f2_fma(wb, hb.r, f2_fma(wa, ha.r, s.c0[p]));
+        s.c1[p] = f2_fma(wb, hb.g, f2_fma(wa, ha.g, s.c1[p]));
+        s.c2[p] = f2_fma(wb, hb.b, f2_fma(wa, ha.b, s.c2[p]));
+        s.D[p] = f2_fma(wb, hb.d, f2_fma(wa, ha.d, s.D[p]));
+        s.T[p] = tb[p];
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        s.last[q] = vb[q] ? pb : (va[q] ? pa : s.last[q]);
+        s.nacc += (va[q] ? 1 : 0) + (vb[q] ? 1 : 0);
+    }
+}
+
 // Walks entries [e0, e1) of a tile's list, which starts at e0, for the lane's pixels until all of
 // the warp's have stopped.  Near: *near is set when a transmittance comes so close to the stop
 // threshold that the same product composed in another order could fall on its other side: two
@@ -312,8 +395,14 @@ __device__ __forceinline__ void walk_list(const FwdArgs &a, uint32_t e0, uint32_
         if (__all_sync(kFull, lane_done)) break;
         const uint32_t g = g_next;
         if (e1 - base > 32u + lane) g_next = a.point_list[base + 32u + lane];
-        const Hit *end = buf + stage_window(a, g, base + lane < e1, base + lane + 1u - e0, bcx, bcy, hw, hh, buf, lane);
-        for (const Hit *h = buf; h != end; ++h) {
+        bool odd;
+        const Hit *end = buf + stage_window(a, g, base + lane < e1, base + lane + 1u - e0, bcx, bcy, hw, hh, buf, lane,
+                                            &odd);
+        const Hit *h = buf;
+        // (windows are all plain or not: asked per pair of records, the test cost what two gained)
+        if (!odd)
+            for (; h + 1 < end; h += 2) blend_two<Q, Near>(h[0], h[1], pxf, s, near);
+        for (; h < end; ++h) {
             if (h->odd != 0.f) blend_hit<Q, true, Near>(*h, pxf, s, near);
             else blend_hit<Q, false, Near>(*h, pxf, s, near);
         }
@@ -327,7 +416,7 @@ __device__ __forceinline__ void walk_list(const FwdArgs &a, uint32_t e0, uint32_
 // window in shared memory, from which every lane reads them (broadcast) and applies them to
 // its Q pixels, which share dx.
 template <int Q>
-__device__ __forceinline__ void pixel_item(const FwdArgs &a, int tile, int sub, Hit *buf, int lane,
+__device__ __forceinline__ void pixel_item(const FwdArgs &a, int tile, int sub, Hit *buf, int *neval, int lane,
                                            unsigned long long &st_eval, unsigned long long &st_acc) {
     constexpr int kItemW = pix_item_w(Q), kItemH = pix_item_h(Q), kRowStep = pix_row_step(Q);
     const TileGeom tg = tile_geom(a, tile);
@@ -341,6 +430,7 @@ __device__ __forceinline__ void pixel_item(const FwdArgs &a, int tile, int sub, 
     const float bcx = (float)(tg.x0 + sx * kItemW) + 0.5f * (kItemW - 1);
     const float bcy = (float)(tg.y0 + sy * kItemH) + 0.5f * (kItemH - 1);
     PixAcc<Q> s;
+    s.neval = neval + lane;
     auto inside = [&](int q) { return q < Q && px < tg.x0 + tg.vw && py0 + kRowStep * q < tg.y0 + tg.vh; };
     auto npy_of = [&](int q) { return inside(q) ? -(float)(py0 + kRowStep * q) : -INFINITY; };
 #pragma unroll
@@ -352,7 +442,7 @@ __device__ __forceinline__ void pixel_item(const FwdArgs &a, int tile, int sub, 
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         s.last[q] = 0;
-        s.neval[q] = (int)(rg.y - rg.x);
+        s.neval[32 * q] = (int)(rg.y - rg.x);
     }
     s.nacc = 0;
     walk_list<Q, false>(a, rg.x, rg.y, pxf, bcx, bcy, 0.5f * (kItemW - 1), 0.5f * (kItemH - 1), buf, lane, s, nullptr);
@@ -365,8 +455,8 @@ __device__ __forceinline__ void pixel_item(const FwdArgs &a, int tile, int sub, 
                 return q & 1 ? u.y : u.x;
             };
             write_pixel(a, tg.v, px, py0 + kRowStep * q, half(s.T[q / 2]), half(s.c0[q / 2]), half(s.c1[q / 2]),
-                        half(s.c2[q / 2]), half(s.D[q / 2]), s.last[q], s.neval[q]);
-            st_eval += (unsigned long long)s.neval[q];
+                        half(s.c2[q / 2]), half(s.D[q / 2]), s.last[q], s.neval[32 * q]);
+            st_eval += (unsigned long long)s.neval[32 * q];
             mlast = max(mlast, s.last[q]);
         }
     }
@@ -1049,7 +1139,8 @@ __device__ __forceinline__ void block_item(const FwdArgs &a, unsigned entry, int
         s.T[0] = f2(1.f, 1.f);
         s.c0[0] = s.c1[0] = s.c2[0] = s.D[0] = f2(0.f, 0.f);
         s.last[0] = s.last[1] = 0;
-        s.neval[0] = s.neval[1] = (int)n;
+        s.neval = reinterpret_cast<int *>(sh.sv) + lane;  // (free until a round is resolved)
+        s.neval[0] = s.neval[32] = (int)n;
         s.nacc = 0;
         bool near = false;
         constexpr float kH = 0.5f * (kGwBlock - 1);
@@ -1065,8 +1156,8 @@ __device__ __forceinline__ void block_item(const FwdArgs &a, unsigned entry, int
                 mlast = s.last[0];
             }
             if (b.in1) {
-                write_pixel(a, b.tg.v, b.px, b.py0 + 4, T.y, c0.y, c1.y, c2.y, D.y, s.last[1], s.neval[1]);
-                st[0] += (unsigned long long)s.neval[1];
+                write_pixel(a, b.tg.v, b.px, b.py0 + 4, T.y, c0.y, c1.y, c2.y, D.y, s.last[1], s.neval[32]);
+                st[0] += (unsigned long long)s.neval[32];
                 mlast = max(mlast, s.last[1]);
             }
             st[1] += (unsigned long long)s.nacc;
@@ -1272,6 +1363,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32) k_forward_gw_merge(FwdArgs a
 template <int Q>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32, Q == 4 ? 3 : 0) k_forward_pixel(FwdArgs a) {
     __shared__ Hit sbuf[kWarpsPerBlock][32];
+    __shared__ int neval[kWarpsPerBlock][32 * 2 * PixAcc<Q>::NP];
     __shared__ unsigned int blk[2];
     if (threadIdx.x == 0) blk[0] = blk[1] = 0u;
     __syncthreads();
@@ -1288,7 +1380,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, Q == 4 ? 3 : 0) k_forward
         const unsigned end = min(first + chunk, num_items);
         for (unsigned it = first; it < end; ++it) {
             const uint2 item = a.items[it - num_gauss];
-            pixel_item<Q>(a, (int)item.x, (int)item.y, buf, lane, st_eval, st_acc);
+            pixel_item<Q>(a, (int)item.x, (int)item.y, buf, neval[threadIdx.x >> 5], lane, st_eval, st_acc);
             ++st_items;
         }
     }
