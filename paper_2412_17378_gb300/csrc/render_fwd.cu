@@ -1119,7 +1119,7 @@ __device__ __noinline__ bool block_composed(const FwdArgs &a, unsigned entry, in
 // too, and the block is written and flagged, which spares its later segments and its merge.
 // The other blocks, and the later segments, are walked with the composed products.  (On a 1080p
 // view of 300k Gaussians under the plan's defaults: 2464 us with pixel-group items alone, 509
-// with the composed walk on every block, 376 with this.)
+// with the composed walk on every block, 376 with this, 327 with two records at a time.)
 __device__ __forceinline__ void block_item(const FwdArgs &a, unsigned entry, int blk, int nb, const SegShared &sh,
                                            int nch, int lane, unsigned long long *st) {
     const uint2 ent = a.gw_ent[entry];
