@@ -532,6 +532,60 @@ __device__ __noinline__ void bwd_pixel_item_wild(const BwdArgs &a, const ItemGeo
     }
 }
 
+// The item of one pixel a lane (Q = 1), the window walked with the scalar pair rule, which holds for
+// every record and gradient: with half of each packed instruction empty the walk of the short
+// lists and few warps that such items are chosen for is slower (256 x 256, 10k Gaussians, captured:
+// the backward call takes 128 us on complete lists and 113 on truncated ones, packed 140 and 127).
+template <bool Extra>
+__device__ __forceinline__ void bwd_pixel_item_one(const BwdArgs &a, const ItemGeom &ig, HitB *buf, int lane) {
+    constexpr int kItemW = pix_item_w(1), kItemH = pix_item_h(1);
+    const int px = ig.x0 + ig.sx * kItemW + (lane % kItemW), py = ig.y0 + ig.sy * kItemH + (lane / kItemW);
+    PixState s = enter_pixel(a, ig, px, py, px < ig.x0 + ig.vw && py < ig.y0 + ig.vh);
+    const uint32_t e0 = ig.e0, first = ig.rg.x, hi = first + (uint32_t)__reduce_max_sync(kFullB, s.nc);
+    const float bcx = (float)(ig.x0 + ig.sx * kItemW) + 0.5f * (kItemW - 1);
+    const float bcy = (float)(ig.y0 + ig.sy * kItemH) + 0.5f * (kItemH - 1);
+    struct Slot {
+        Rec r;
+        uint32_t idx;
+        int pos;
+        float2 pad;
+    };
+    static_assert(sizeof(Slot) <= sizeof(HitB), "a window slot");
+    Slot *win = reinterpret_cast<Slot *>(buf);
+    // the point-list index of the lane's next entry, loaded a window ahead
+    uint32_t g_next = hi > e0 + lane ? a.point_list[hi - 1u - lane] : 0u;
+    for (uint32_t top = hi; top > e0; top -= min(32u, top - e0)) {
+        const uint32_t g = g_next;
+        bool hit = false;
+        Rec r;
+        if (top > e0 + lane) {
+            if ((long long)g < a.N) {
+                r = a.recs[g];
+                hit = !block_misses(r.a, r.b, bcx, bcy, 0.5f * (kItemW - 1), 0.5f * (kItemH - 1));
+            } else {
+                raise_check(a.ctrl, BGS_CHECK_INDEX);  // a transparent entry
+            }
+        }
+        if (top > e0 + 32u + lane) g_next = a.point_list[top - 33u - lane];
+        const unsigned live = __ballot_sync(kFullB, hit);
+        if (hit) {
+            Slot *w = win + __popc(live & ((1u << lane) - 1u));
+            w->r = r;
+            w->idx = g;
+            w->pos = (int)(top - 1u - lane - first);
+        }
+        __syncwarp();
+        const Slot *end = win + __popc(live);
+        for (const Slot *w = win; w != end; ++w) {
+            const PairX x = pair_x(w->r.a, (float)px);
+            PairSums sums = zero_sums();
+            const bool any = pair_backward<Extra>(w->r, x, (float)py, w->pos < s.nc, s, sums);
+            if (__any_sync(kFullB, any)) warp_reduce_red<Extra>(sums, x.dx, a.grad_acc + 12ull * w->idx, lane);
+        }
+        __syncwarp();
+    }
+}
+
 // The walk is latency-bound (dependent FP32 chains, shuffle trees): with colour-only output
 // gradients and up to 4 rows per lane the kernel fits 64 registers, so 4 blocks (32 warps)
 // stay resident per SM instead of 3.  The other variants would spill there: 3 blocks for
@@ -556,7 +610,8 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (Q <= 4 && !Extra) ? 4 : (Q <=
         for (unsigned it = first; it < end; ++it) {
             const uint2 item = a.items[it];
             const ItemGeom ig = item_geom<Q>(a, (int)item.x, (int)item.y, L);
-            if (!bwd_pixel_item<Q, Extra>(a, ig, buf, lane)) bwd_pixel_item_wild<Q, Extra>(a, ig, lane);
+            if constexpr (Q == 1) bwd_pixel_item_one<Extra>(a, ig, buf, lane);
+            else if (!bwd_pixel_item<Q, Extra>(a, ig, buf, lane)) bwd_pixel_item_wild<Q, Extra>(a, ig, lane);
             ++st_items;
         }
     }
